@@ -48,6 +48,7 @@ FLOP_PER_TRI = 45.0
 SM_COUNT = 152
 FP32_LANES_PER_SM = 128
 NODE_BYTES, TRI_BYTES = 64, 48        # 4-wide BVH node (quantised child boxes); three float4 vertices
+CELL_BYTES, CELL_TRI_BYTES = 4, 52    # uniform grid: a cell's word; a list entry and three float4 vertices
 L2_FLUSH_BYTES = 512 << 20
 
 
@@ -76,7 +77,7 @@ def workload_config(name, n_hist):
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("transport.cu", "wavefront.cu", "transport_common.cuh", "device_common.cuh"):
+    for f in ("transport.cu", "wavefront.cu", "transport_common.cuh", "device_common.cuh", "grid.cuh", "grid.cu"):
         with open(os.path.join(ROOT, "paper_2605_25963_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -329,6 +330,15 @@ def measure_forms(dev, scale=1.0):
     return out
 
 
+def structure_bytes(nodes, boxes, tris):
+    """Algorithmic bytes of the traversal: node and triangle records, or cell words, list
+    entries and triangle records where the run walks grids (each cell counts as one node
+    and one box; a tree's nodes hold two boxes and more)."""
+    if boxes == nodes:
+        return CELL_BYTES * nodes + CELL_TRI_BYTES * tris
+    return NODE_BYTES * nodes + TRI_BYTES * tris
+
+
 def stress_roofline(bvh, mats, items, dev):
     """Roofline of the trace kernel on the stress workload: the one batched plan
     timed again with a CUDA event pair around every kernel (host-issued
@@ -343,6 +353,7 @@ def stress_roofline(bvh, mats, items, dev):
     p.launch()
     st = p.kernel_stats(reset=True)
     res, _, _, _ = p.results(want_spectra=False)
+    queued = sum(p.queue_sizes())
     del p
     _, nodes, tris, _, boxes = api.gadep_count_work(bvh, mats, api.make_instances(items), api.make_opts())
     segs = sum(r["n_segments"] for r in res)
@@ -351,13 +362,13 @@ def stress_roofline(bvh, mats, items, dev):
     if not nl:
         return None
     flops = FLOP_PER_BOX * boxes + FLOP_PER_TRI * tris
-    bytes_ = NODE_BYTES * nodes + TRI_BYTES * tris
+    bytes_ = structure_bytes(nodes, boxes, tris)
     sm_max = measured_peaks().get("sm_max_mhz") or 2070.0
     peak = SM_COUNT * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     achieved = flops / (ms / 1e3) / 1e12
     hbm = measured_peaks().get("hbm_gbs")
     return {"bound": "alu", "kernel": "trace", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": achieved / peak, "traffic": recorded_traffic("stress", "trace", queries / nl),
+            "frac": achieved / peak, "traffic": recorded_traffic("stress", "trace", queued / nl),
             "launches": nl, "avg_launch_ms": ms / nl, "flop_per_launch": flops / nl,
             "node_tri_bytes_gbs": bytes_ / (ms / 1e3) / 1e9, "hbm_peak_gbs": hbm,
             "per_query": {"nodes": nodes / max(queries, 1), "boxes": boxes / max(queries, 1),
@@ -589,7 +600,8 @@ def main():
     for f, E in zip(fepe, cfg["energies"]):
         f["E_keV"] = E
 
-    qlog = [p.queue_sizes() for p in plans] if args.queue_log else None
+    qlog = [p.queue_sizes() for p in plans]
+    queued = sum(sum(q) for q in qlog)      # photons the trace launches of one step served
     # algorithmic work of one step (instrumented copy of the kernel, untimed)
     nodes = tris = relocated = boxes = 0
     for i, E in enumerate(cfg["energies"]):
@@ -624,7 +636,7 @@ def main():
     queries = segs - sum(f["culled"] for f in fepe)
     # algorithmic node and triangle bytes of the traversal (64 B per node visit, 48 B per
     # triangle test), served by L1 and L2, per second of the dominant kernel
-    l1l2_gbs = (NODE_BYTES * nodes + TRI_BYTES * tris) * args.steps / (dom_ms / 1e3) / 1e9
+    l1l2_gbs = structure_bytes(nodes, boxes, tris) * args.steps / (dom_ms / 1e3) / 1e9
     # the timed plans hold the mesh's cached wavefront buffers; release them so the
     # public-API calls below find the cache free, as a caller's successive runs do
     n_plans, shape = len(plans), plans[0].shape()
@@ -687,7 +699,7 @@ def main():
             "roofline": {"bound": "alu", "kernel": dom, "achieved": achieved_tflops, "peak": peak_tflops,
                          "unit": "TFLOP/s", "frac": achieved_tflops / peak_tflops,
                          "traffic": recorded_traffic(args.workload, dom,
-                                                     queries * args.steps / max(dom_launches, 1)),
+                                                     queued * args.steps / max(dom_launches, 1)),
                          "launches": dom_launches, "avg_launch_ms": dom_ms / max(dom_launches, 1),
                          "flop_per_launch": flops_per_step * args.steps / max(dom_launches, 1),
                          "peak_note": "FP32 non-tensor: %d SMs x %d lanes x 2 x %.0f MHz (derived)" % (
@@ -714,7 +726,7 @@ def main():
         }
         if sweep is not None:
             line["mesh_sweep"] = sweep
-        if qlog is not None:
+        if args.queue_log:
             line["queue_sizes"] = qlog
         print(json.dumps(line), flush=True)
     if dist is not None:

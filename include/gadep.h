@@ -475,6 +475,8 @@ gadep_status gadep_plan_queue_sizes(gadep_plan *p, uint32_t *out, int32_t max, i
  * counted) and triangles tested, summed over all segment queries, and the number
  * of queries that found no surface in their region's tree and were relocated
  * through the tree of every triangle (photons a rounding error past a boundary).
+ * Where the run walks the regions' uniform grids instead of the trees, the grid
+ * cells visited count as nodes and as boxes alike.
  * `relocated` and `boxes_tested` may be NULL.  Runs an instrumented copy of the
  * transport kernels; used to turn the measured time into algorithmic bytes and
  * FLOPs per query.  results: host [n_inst]. */

@@ -23,7 +23,7 @@ LIB = os.path.join(OUT_DIR, "libgadep.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 CXX_SOURCES = ["detmesh.cpp", "geometry.cpp", "xs.cpp", "bvh.cpp"]
-CU_SOURCES = ["transport.cu", "wavefront.cu"]
+CU_SOURCES = ["transport.cu", "wavefront.cu", "grid.cu"]
 
 
 def _cuda_home() -> str:

@@ -103,10 +103,17 @@ struct gadep_bvh {
     gadep_bvh_stats stats{};
     void *d_nodes = nullptr, *d_tris = nullptr, *d_tri_orig = nullptr, *d_regions = nullptr,
          *d_planes = nullptr;
+    // uniform grids of the segment queries (grid.cu): one block of descriptors, cells
+    // and triangle records, and the cells' lists; null when none were built
+    void *d_grid = nullptr, *d_grid_list = nullptr;
+    size_t grid_cells = 0, grid_tris = 0;   // byte offsets within d_grid
+    float grid_safe = 0.0f;                 // origins the grids serve: components within this
 };
 
 namespace gadep {
 std::vector<std::vector<int32_t>> region_triangle_sets(const MeshData &g);
 gadep_status upload_bvh(gadep_bvh *b);
 void free_bvh_device(gadep_bvh *b);
+gadep_status grid_build(gadep_bvh *b);
+void grid_free(gadep_bvh *b);
 }  // namespace gadep

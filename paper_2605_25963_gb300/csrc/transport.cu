@@ -46,8 +46,9 @@ gadep_status build_bvh_host(const detmesh_mesh *m, const gadep_bvh_opts &o, gade
 
 namespace dev {
 // EM: charged-particle tracks (e_model 1), a separate instantiation so that the
-// photon-only kernels keep their registers.
-template <bool GRAD, bool COUNT, bool EM>
+// photon-only kernels keep their registers.  GRID: the queries walk the regions'
+// grids (grid.cuh) instead of their trees.
+template <bool GRAD, bool COUNT, bool EM, bool GRID>
 // 4 blocks of 256 threads per SM (64 registers): measured faster than 2 or 3
 // blocks despite the register spills, as the traversal is latency bound.
 __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsigned long long *counters)
@@ -167,21 +168,30 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                 bool entering = false;
                 // region record: material slot, active | (group + 1) << 1, parent, tree root
                 int4 R = s_reg[region];
-                int hit = traverse<COUNT>(P.nodes, P.tris, P.planes, R.w, ox, oy, oz, dx, dy, dz, t_cur, last_tri,
-                                          t_hit, entering, herr, ts);
-                if (hit < 0 && region != 0 && !(herr & ERR_STACK)) {
+                // hit: a mesh triangle for the grids, a triangle slot of the tree otherwise
+                int hit = -1;
+                bool reloc = false, by_tree = !GRID;
+                while (true) {
+                    if (!by_tree) {
+                        hit = grid_query<COUNT, true>(P.grid, P.planes, reloc ? P.grid.all : region, ox, oy, oz, dx, dy, dz,
+                                                t_cur, last_tri, t_hit, entering, by_tree, ts);
+                        if (by_tree) continue;          // left to the tree
+                    } else {
+                        hit = traverse<COUNT>(P.nodes, P.tris, P.planes, reloc ? P.root_all : R.w, ox, oy, oz, dx, dy,
+                                              dz, t_cur, last_tri, t_hit, entering, herr, ts);
+                    }
+                    if (reloc || hit >= 0 || region == 0 || (herr & ERR_STACK)) break;
                     // Inside a solid every ray meets that solid's boundary, so the
                     // photon actually sits a rounding error past it (an interaction
                     // point computed in FP32 right at a surface).  Relocate by the
                     // nearest surface of the whole mesh and the nesting-tree rule;
                     // with no surface ahead it is outside every solid.
-                    hit = traverse<COUNT>(P.nodes, P.tris, P.planes, P.root_all, ox, oy, oz, dx, dy, dz, t_cur, last_tri,
-                                          t_hit, entering, herr, ts);
+                    reloc = true;
                     if (COUNT) ts.relocated++;
-                    if (hit < 0) {
-                        region = 0;
-                        R = s_reg[0];       // the segment runs in the world
-                    }
+                }
+                if (reloc && hit < 0) {
+                    region = 0;
+                    R = s_reg[0];       // the segment runs in the world
                 }
                 const int group = (R.y >> 1) - 1;
                 float pe = 0.0f, co = 0.0f, pa = 0.0f;
@@ -261,7 +271,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                     if (R.y & 1) edep += dep;
                     dep_all += dep;
                     if (eT > 0.0f && !herr)
-                        e_track<COUNT>(P, s_reg, P.inst[inst].scale, px, py, pz, eux, euy, euz, eT, ew, region, edep,
+                        e_track<COUNT, GRID>(P, s_reg, P.inst[inst].scale, px, py, pz, eux, euy, euz, eT, ew, region, edep,
                                        dep_all, esc, herr, ts);
                     if (herr) {
                         finished = true;
@@ -298,8 +308,9 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                     lam -= mu * len;
                     if (GRAD && group >= 0 && group < 4) score[group] -= mu_unit * len;
                     t_cur = t_hit;
-                    last_tri = __float_as_int(__ldg(&P.tris[3 * hit + 1].w));   // mesh triangle id
-                    const int treg = __float_as_int(__ldg(&P.tris[3 * hit].w));
+                    // mesh triangle id, region of its solid
+                    last_tri = by_tree ? __float_as_int(__ldg(&P.tris[3 * hit + 1].w)) : hit;
+                    const int treg = __float_as_int(__ldg(by_tree ? &P.tris[3 * hit].w : &P.grid.tris[3 * hit].w));
                     region = entering ? treg : s_reg[treg].z;
                 }
             }
@@ -492,7 +503,7 @@ gadep_status upload_bvh(gadep_bvh *b)
         (e = cudaMemcpy(b->d_planes, b->planes.data(), b->planes.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->d_regions, roots.data(), nr * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
         return cuda_fail(e, "gadep_bvh_build: upload");
-    return GADEP_OK;
+    return grid_build(b);
 }
 
 void free_bvh_device(gadep_bvh *b)
@@ -504,6 +515,7 @@ void free_bvh_device(gadep_bvh *b)
     cudaFree(b->plan_scratch);
     b->plan_scratch = nullptr;
     b->plan_scratch_bytes = 0;
+    grid_free(b);
     cudaFree(b->d_nodes);
     cudaFree(b->d_tris);
     cudaFree(b->d_regions);
@@ -566,14 +578,18 @@ gadep_status check_opts(const gadep_opts *o)
     return GADEP_OK;
 }
 
-template <bool GRAD, bool COUNT, bool EM>
-void *kernel_ptr() { return (void *)gadep::dev::transport_kernel<GRAD, COUNT, EM>; }
-
-void *pick_kernel(bool grad, bool count, bool em)
+template <bool GRID>
+void *kernel_of(bool grad, bool count, bool em)
 {
-    if (grad) return count ? kernel_ptr<true, true, false>() : kernel_ptr<true, false, false>();
-    if (em) return count ? kernel_ptr<false, true, true>() : kernel_ptr<false, false, true>();
-    return count ? kernel_ptr<false, true, false>() : kernel_ptr<false, false, false>();
+    using namespace gadep::dev;
+    if (grad) return count ? (void *)transport_kernel<true, true, false, GRID> : (void *)transport_kernel<true, false, false, GRID>;
+    if (em) return count ? (void *)transport_kernel<false, true, true, GRID> : (void *)transport_kernel<false, false, true, GRID>;
+    return count ? (void *)transport_kernel<false, true, false, GRID> : (void *)transport_kernel<false, false, false, GRID>;
+}
+
+void *pick_kernel(bool grad, bool count, bool em, bool grid)
+{
+    return grid ? kernel_of<true>(grad, count, em) : kernel_of<false>(grad, count, em);
 }
 
 }  // namespace
@@ -758,6 +774,28 @@ double hit_fraction(const dev::InstDev &d, const float lo[3], const float hi[3])
     return (double)hit / ((double)n_dir * n_pos);
 }
 
+// Meshes from this size on run the megakernel on the grids.  On the smallest the tree is a
+// few nodes: ms per run, tree / grids: 192 triangles 0.200 / 0.205, 3,456 triangles 0.81 /
+// 0.81, coax geometry 20,088 triangles 1e6 histories 2.13 / 1.41, 3e5 histories 1.12 /
+// 0.62, with charged-particle tracks 2.21 / 1.48, 216,684 triangles 2.36 / 2.14.
+constexpr int kMegaGridMinTri = 8192;
+
+// The grids for a run of these instances (desc null: the tree serves it).  Every birth
+// point has to lie where the grids' margins cover the rounding of positions along its rays.
+dev::GridSet grid_of(const gadep_bvh *b, const dev::InstDev *inst, int n_inst, int min_tri)
+{
+    dev::GridSet g = grid_set(b);
+    if (g.n_tri < min_tri) g.desc = nullptr;
+    for (int i = 0; i < n_inst; ++i) {
+        const dev::InstDev &d = inst[i];
+        const float far = std::max(std::fabs(d.px), std::max(std::fabs(d.py), std::fabs(d.pz)));
+        const float ext = (d.src_kind == GADEP_SRC_DISK || d.src_kind == GADEP_SRC_PRISM ? d.radius : 0.0f) +
+                          (d.src_kind == GADEP_SRC_PRISM ? d.height : 0.0f);
+        if (!(far + ext < b->grid_safe)) g.desc = nullptr;
+    }
+    return g;
+}
+
 gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t n_inst,
                          const gadep_instance *inst, const gadep_opts *opts, bool grad, bool count,
                          gadep_plan **out)
@@ -885,7 +923,8 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
         gadep_plan_destroy(p);
         return fail(GADEP_E_INVAL, "plan: tables need %zu bytes of shared memory, the device has %d", smem, dev_smem);
     }
-    void *kfn = pick_kernel(grad, count, opts->e_model == 1);
+    p->P.grid = grid_of(b, p->inst.data(), n_inst, kMegaGridMinTri);
+    void *kfn = pick_kernel(grad, count, opts->e_model == 1, p->P.grid.desc != nullptr);
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) { gadep_plan_destroy(p); return cuda_fail(e, "plan: cudaFuncSetAttribute"); }
     int bps = 0;
@@ -1081,15 +1120,11 @@ gadep_status plan_launch(gadep_plan *p, uint32_t *spectra_dev, float *edep_trace
     if (P.total == 0) return GADEP_OK;
     if (p->wf) return wavefront_run(p->wf, P, p->grad, p->count, p->d_counters, &p->timer, s, p->wf_slots);
     p->timer.before(s);
-    if (p->grad) {
-        if (p->count) dev::transport_kernel<true, true, false><<<p->grid, p->block, p->smem, s>>>(P, p->d_counters);
-        else dev::transport_kernel<true, false, false><<<p->grid, p->block, p->smem, s>>>(P, p->d_counters);
-    } else if (P.e_model) {
-        if (p->count) dev::transport_kernel<false, true, true><<<p->grid, p->block, p->smem, s>>>(P, p->d_counters);
-        else dev::transport_kernel<false, false, true><<<p->grid, p->block, p->smem, s>>>(P, p->d_counters);
-    } else {
-        if (p->count) dev::transport_kernel<false, true, false><<<p->grid, p->block, p->smem, s>>>(P, p->d_counters);
-        else dev::transport_kernel<false, false, false><<<p->grid, p->block, p->smem, s>>>(P, p->d_counters);
+    {
+        void *args[] = { &P, &p->d_counters };
+        e = cudaLaunchKernel(pick_kernel(p->grad, p->count, P.e_model != 0, P.grid.desc != nullptr), dim3(p->grid),
+                             dim3(p->block), args, (size_t)p->smem, s);
+        if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "plan launch: kernel"); }
     }
     p->timer.after(KK_MEGA, s);
     e = cudaGetLastError();
@@ -1542,7 +1577,8 @@ extern "C" gadep_status gadep_run_noalloc(const gadep_bvh *b, const gadep_materi
     cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, b->device);
     if (smem > (size_t)dev_smem) return fail(GADEP_E_INVAL, "gadep_run_noalloc: tables need too much shared memory");
-    void *kfn = (void *)dev::transport_kernel<false, false, false>;
+    const dev::GridSet grid = grid_of(b, &d, 1, kMegaGridMinTri);
+    void *kfn = pick_kernel(false, false, false, grid.desc != nullptr);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, block, smem);
     if (e == cudaSuccess && bps < 1) return fail(GADEP_E_CUDA, "gadep_run_noalloc: kernel does not fit on the device");
@@ -1594,9 +1630,13 @@ extern "C" gadep_status gadep_run_noalloc(const gadep_bvh *b, const gadep_materi
     P.n_stripes = 1;                       // the one tally record of the scratch array
     P.root_all = b->root_all;
     gadep::scene_box(b, P.root_lo, P.root_hi);
-    if (n_hist > 0)
-        dev::transport_kernel<false, false, false><<<n_sm * bps, block, smem, s>>>(P, S->counters);
-    e = cudaGetLastError();
+    P.grid = grid;
+    if (n_hist > 0) {
+        unsigned long long *counters = S->counters;
+        void *args[] = { &P, &counters };
+        e = cudaLaunchKernel(kfn, dim3(n_sm * bps), dim3(block), args, smem, s);
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "gadep_run_noalloc: launch");
     // tallies back to the host, finalise
     dev::TallyDev t;

@@ -7,6 +7,7 @@
 
 #include "device_common.cuh"
 #include "gadep.h"
+#include "grid.cuh"
 
 namespace gadep {
 namespace dev {
@@ -60,6 +61,7 @@ struct Params {
     const float *erange;                // [n_mat][e_n]
     int e_model, e_n;
     float e_T_min, e_lnT_min, e_inv_dlnT;
+    GridSet grid;                       // desc null: the queries take the tree
 };
 
 // Slab test of the ray (t >= 0) against an axis-aligned box.
@@ -257,7 +259,7 @@ constexpr int kMaxTrackCrossings = 256;
 // cross it with the T' of range R_m(T) - s L and deposit T - T' in the region.
 // Below e_T_min the rest is deposited where they are; vacuum takes nothing; what
 // leaves the mesh escapes.  Active deposits go to edep, all to dep_all.
-template <bool COUNT>
+template <bool COUNT, bool GRID>
 __device__ void e_track(const Params &P, const int4 *s_reg, const float *scale, float px, float py, float pz,
                         float ux, float uy, float uz, float T, float w, int region, float &edep, float &dep_all,
                         float &esc, uint32_t &herr, TravStats &ts)
@@ -277,20 +279,26 @@ __device__ void e_track(const Params &P, const int4 *s_reg, const float *scale, 
         const float reach = rn / sc;
         float t_hit = INFINITY;
         bool entering = false;
-        int hit = traverse<COUNT>(P.nodes, P.tris, P.planes, R.w, px, py, pz, ux, uy, uz, t_cur, last, t_hit,
-                                  entering, herr, ts, t_cur + reach);
-        if (herr & ERR_STACK) return;
-        if (hit < 0 && reach < INFINITY) {         // stops in this region
-            dep_all += w * T;
-            if (R.y & 1) edep += w * T;
-            return;
-        }
-        if (hit < 0 && region != 0) {
+        int hit;
+        bool left;                                 // either triangle of an edge serves a track
+        for (bool reloc = false;; reloc = true) {
+            const float t_max = reloc ? INFINITY : t_cur + reach;
+            if (GRID)
+                hit = grid_query<COUNT, false>(P.grid, P.planes, reloc ? P.grid.all : region, px, py, pz, ux, uy, uz, t_cur,
+                                        last, t_hit, entering, left, ts, t_max);
+            else
+                hit = traverse<COUNT>(P.nodes, P.tris, P.planes, reloc ? P.root_all : R.w, px, py, pz, ux, uy, uz,
+                                      t_cur, last, t_hit, entering, herr, ts, t_max);
+            if (herr & ERR_STACK) return;
+            if (reloc || hit >= 0) break;
+            if (reach < INFINITY) {                // stops in this region
+                dep_all += w * T;
+                if (R.y & 1) edep += w * T;
+                return;
+            }
+            if (region == 0) break;
             // vacuum inside a solid with no surface ahead: the start sits a rounding
             // error past a boundary; relocate by the nearest surface of the mesh
-            hit = traverse<COUNT>(P.nodes, P.tris, P.planes, P.root_all, px, py, pz, ux, uy, uz, t_cur, last,
-                                  t_hit, entering, herr, ts);
-            if (herr & ERR_STACK) return;
         }
         if (hit < 0) {                             // leaves the mesh
             esc += w * T;
@@ -302,8 +310,8 @@ __device__ void e_track(const Params &P, const int4 *s_reg, const float *scale, 
         if (R.y & 1) edep += w * (T - T2);
         T = T2;
         t_cur = t_hit;
-        last = __float_as_int(__ldg(&P.tris[3 * hit + 1].w));
-        const int treg = __float_as_int(__ldg(&P.tris[3 * hit].w));
+        last = GRID ? hit : __float_as_int(__ldg(&P.tris[3 * hit + 1].w));
+        const int treg = __float_as_int(__ldg(GRID ? &P.grid.tris[3 * hit].w : &P.tris[3 * hit].w));
         region = entering ? treg : s_reg[treg].z;
     }
     herr |= ERR_STEPCAP;
@@ -376,6 +384,7 @@ struct KernelTimer {
 // spawn / sort / trace / physics / gen / ctrl kernels per iteration.
 struct WavefrontBuffers;
 constexpr int kWavefrontMaxInstances = 1024;   // block tallies live in shared memory
+dev::GridSet grid_set(const gadep_bvh *b);
 gadep_status wavefront_create(int device, int slots, bool grad, WavefrontBuffers **out);
 void wavefront_destroy(WavefrontBuffers *w);
 // slots: photon slots the run keeps in flight (at most the buffers' capacity; 0 =

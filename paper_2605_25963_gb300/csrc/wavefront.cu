@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
                             tr.tag = (uint32_t)region | ((uint32_t)inst << 8);
                         } else {
                             float e_esc = 0.0f;
-                            e_track<COUNT>(P, s_reg, I.scale, px, py, pz, eux, euy, euz, eT, ew, region, edep,
+                            e_track<COUNT, false>(P, s_reg, I.scale, px, py, pz, eux, euy, euz, eT, ew, region, edep,
                                            dep_all, e_esc, herr, ts);
                             esc_now += e_esc;
                         }
@@ -1230,7 +1230,7 @@ __global__ void __launch_bounds__(256) etrack_kernel(const Params P, State S, un
         const int region = (int)(t.tag & 255u), inst = (int)(t.tag >> 8);
         float edep = 0.0f, dep_all = 0.0f, esc = 0.0f;
         uint32_t herr = 0;
-        e_track<COUNT>(P, s_reg, P.inst[inst].scale, t.p.x, t.p.y, t.p.z, t.u.x, t.u.y, t.u.z, t.p.w, t.u.w, region,
+        e_track<COUNT, false>(P, s_reg, P.inst[inst].scale, t.p.x, t.p.y, t.p.z, t.u.x, t.u.y, t.u.z, t.p.w, t.u.w, region,
                        edep, dep_all, esc, herr, ts);
         SlotA &a = S.slot[t.slot].a;
         uint4 u = a.u;
