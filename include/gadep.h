@@ -464,7 +464,8 @@ gadep_status gadep_plan_set_timing(gadep_plan *p, int32_t on);
 gadep_status gadep_plan_kernel_stats(gadep_plan *p, gadep_kernel_stats *out, int32_t reset);
 
 /* Trace queue size of each wavefront iteration of the plan's last launch, in
- * order (the queries its trace kernel launches served), for measurements that
+ * order (the photons its trace kernel launches served, one query each, or one
+ * flight where the trace kernel applies the boundary crossings itself), for measurements that
  * need the work of individual launches (no counterpart in the paper).  out: host
  * [max]; *n: entries written (0 for a megakernel plan; the log holds the first
  * 8192 iterations).  Synchronises `stream`. */

@@ -960,6 +960,25 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
                                    "2^23 - 1 triangles", kWavefrontMaxInstances);
     }
     if (variant == GADEP_VARIANT_WAVEFRONT) {
+        bool one_point = true;          // every history starts at one and the same point
+        for (const dev::InstDev &d : p->inst)
+            one_point = one_point && d.src_kind == GADEP_SRC_POINT && d.px == p->inst[0].px &&
+                        d.py == p->inst[0].py && d.pz == p->inst[0].pz;
+        const bool many = reaching >= (double)(1u << 20);
+        // The trace kernel walks the grids of middling meshes.  Measured per run (ms, tree /
+        // grids, both with sorted births): 20,088 triangles, 1332 keV, 2.5e7 reaching 35.1 /
+        // 32.5, 59.5 keV 17.6 / 14.3, 662 keV 5e6 reaching 9.88 / 9.10, 1.5e6 reaching 5.17 /
+        // 5.13, 5e5 reaching 3.57 / 3.72; gradients from a volume, 4.8e6 histories 7.97 / 7.56,
+        // 2.4e6 5.59 / 5.67; with charged-particle tracks, 1.25e6 reaching 8.3 / 5.8, 3e5
+        // reaching 5.9 / 4.2 (3,456 triangles 7.0 / 5.0).  On the smallest meshes
+        // the tree is a few nodes (192 triangles 2.80 / 3.37), on large ones the cells miss
+        // the caches (25,112 triangles, 1.5e6 reaching 5.38 / 5.52; 76,280 triangles, 7.5e6
+        // reaching 14.5 / 15.8); a plain volume source gains 2 % at best.
+        const int n_tri = b->geo.n_tri();
+        const bool walks = electrons ? n_tri >= 2048 && n_tri <= 49152
+                                     : ((one_point && many) || (grad && reaching >= (double)(1u << 22))) &&
+                                           n_tri >= 4096 && n_tri <= 24576;
+        p->P.grid = walks ? grid_of(b, p->inst.data(), n_inst, 1) : dev::GridSet{};
         int slots = opts->wf_slots;
         if (slots <= 0) {
             // every photon that reaches the scene in flight at once where that fits:

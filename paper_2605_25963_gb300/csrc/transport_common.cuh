@@ -202,11 +202,11 @@ __device__ __forceinline__ void iso_dir(Stream &rng, uint32_t k0, uint32_t k1, f
     dx = s * cp; dy = s * sp; dz = c;
 }
 
-// Interpolated attenuation (pe, compton, pair) of a staged material at energy E.
-__device__ __forceinline__ void mu_at(const float4 *tab, int n_grid, float lnE_min, float inv_dl,
-                                      float E, float &pe, float &co, float &pa)
+// Interpolated attenuation (pe, compton, pair) of a staged material at energy E, whose
+// place on the tables' grid is g.
+__device__ __forceinline__ void mu_on_grid(const float4 *tab, int n_grid, float g, float E, float &pe, float &co,
+                                           float &pa)
 {
-    const float g = (logf(E) - lnE_min) * inv_dl;
     int k = (int)floorf(g);
     k = min(max(k, 0), n_grid - 2);
     const float f = fminf(fmaxf(g - (float)k, 0.0f), 1.0f);
@@ -214,6 +214,12 @@ __device__ __forceinline__ void mu_at(const float4 *tab, int n_grid, float lnE_m
     pe = fmaf(f, b.x - a.x, a.x);
     co = fmaf(f, b.y - a.y, a.y);
     pa = E > kTwoMeC2 ? fmaf(f, b.z - a.z, a.z) : 0.0f;
+}
+
+__device__ __forceinline__ void mu_at(const float4 *tab, int n_grid, float lnE_min, float inv_dl,
+                                      float E, float &pe, float &co, float &pa)
+{
+    mu_on_grid(tab, n_grid, (logf(E) - lnE_min) * inv_dl, E, pe, co, pa);
 }
 
 // CSDA range (mm, unit density) of staged material m at kinetic energy T >= e_T_min:

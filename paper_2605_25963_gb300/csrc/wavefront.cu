@@ -12,7 +12,9 @@
 //   trace    lean persistent traversal: warps claim chunks of the queue, lanes
 //            that finish a query take the next entry as soon as too few lanes of
 //            the warp are still traversing (dynamic fetch), so the warp is not
-//            held by its longest ray; the hit is stored by queue position;
+//            held by its longest ray; the hit is stored by queue position.  On
+//            middling meshes a second form walks uniform grids instead of the trees
+//            and applies the boundary crossings of a flight on the way;
 //   physics  one thread per queued photon applies the segment: free flight,
 //            boundary crossing (nesting-tree rule), interaction or escape, and the
 //            end-of-history tally; survivors go to the next trace queue, finished
@@ -72,13 +74,16 @@ struct __align__(16) Hit {      // by queue position, written by trace
     float t;
     int tri;                    // mesh triangle id, -1 = nothing ahead
     int region;                 // region of the triangle's solid
-    int entering;               // 1 entering, 0 leaving, -2 traversal stack overflow,
-                                // kBeyond: no surface before the sampled interaction point;
-                                // + kRelocated when the hit (or tri -1: none) came from the
-                                // tree of every triangle (relocation, see trace_kernel)
+    int code;                   // low four bits, less kCodeBias: 1 entering, 0 leaving, -2
+                                // traversal stack overflow, kBeyond: no surface before the
+                                // sampled interaction point; + kRelocated when the hit (or tri
+                                // -1: none) came from the tree of every triangle (relocation,
+                                // see trace_kernel).  Above: boundary crossings already applied
 };
 constexpr int kBeyond = -3;
 constexpr int kRelocated = 4;
+constexpr int kCodeBias = 8, kCodeBits = 4;
+constexpr int kMaxCrossed = 1 << 20;
 static_assert(sizeof(Slot) == 64 && sizeof(SlotA) == 32, "slot record: two 32-byte DRAM sectors");
 // A charged-particle track (e_model 1) whose history goes on after the physics
 // visit that set it going: traced by etrack_kernel before the slot's next visit.
@@ -323,6 +328,7 @@ struct Ctrl {
     unsigned long long max_iter;
     unsigned int t_count;          // deferred charged-particle tracks of this iteration
     unsigned int qlog_n;           // iterations whose queue size is in the log
+    unsigned int n_left;           // queries of this iteration that the grids left to the tree
 };
 
 struct State {
@@ -344,6 +350,7 @@ struct State {
     unsigned long long pend_mask;  // ring size - 1 (a power of two)
     unsigned long long gen_target; // ring fill at which gen stops claiming ids
     Ctrl *ctrl;
+    unsigned int *left;            // queue positions of the queries left to the tree
     unsigned int *qlog;            // trace queue size of each iteration (the first kQueueLog)
     int slots;
 };
@@ -422,6 +429,7 @@ __global__ void init_kernel(State S, unsigned long long max_iter)
         c.max_iter = max_iter;
         c.t_count = 0;
         c.qlog_n = 0;
+        c.n_left = 0;
     }
 }
 
@@ -449,6 +457,7 @@ __device__ __forceinline__ void ctrl_step(Ctrl &c, int cur, unsigned long long t
     c.q_count[cur] = 0;
     c.t_count = 0;                 // etrack has run
     c.trace_head = 0;
+    c.n_left = 0;
     c.gen_live = avail - filled;
     c.iter++;
     if (work >= total && avail == 0 && n_alive == 0) c.done = 1;
@@ -858,9 +867,9 @@ __global__ void __launch_bounds__(256, 4) trace_kernel(const Params P, State S, 
                                           t_min)
                                 : INFINITY;
                 h.region = best >= 0 ? __float_as_int(__ldg(&tris[3 * best].w)) : 0;
-                h.entering = (err & ERR_STACK) ? -2
-                           : (best >= 0 ? (ent ? 1 : 0) + (reloc ? kRelocated : 0)
-                                        : (reloc ? kRelocated : (bounded ? kBeyond : 0)));
+                h.code = kCodeBias + ((err & ERR_STACK) ? -2
+                                      : (best >= 0 ? (ent ? 1 : 0) + (reloc ? kRelocated : 0)
+                                                   : (reloc ? kRelocated : (bounded ? kBeyond : 0))));
                 S.hit[qidx] = h;
                 err = 0;
                 has = false;
@@ -875,13 +884,306 @@ __global__ void __launch_bounds__(256, 4) trace_kernel(const Params P, State S, 
     }
 }
 
+// The same queries through the regions' grids (grid.cuh), and the boundary crossings
+// between them: a photon that meets a surface before its interaction point goes on in
+// the region behind it at once, with physics' own arithmetic, so that physics sees a
+// photon once per flight and not once per segment.
+// Bound by instruction issue (70 % of issue slots, 16 of 32 lanes, L1 data pipe 71 %, DRAM
+// idle), so the warp's lanes are kept together: at any time the warp does the one thing
+// that enough of its lanes wait for -- a step from cell to cell, a triangle test, or the
+// ends of queries and the fetch of new photons.  Lane by lane, without the votes, 8.8 of
+// 32 lanes had work (trace 34.2 ms per 1e8 histories at 1332 keV, 31.5 with them); tests
+// shared out over the warp through shared memory reached 26 lanes but paid as much for
+// finding their rays (32.9 ms).  With the crossings physics takes 3.0 ms instead of 8.1
+// and the sort 0.8 instead of 2.3.
+constexpr int kStepMin = 6, kTestMin = 10, kServeMin = 14, kFetchMin = 6;
+// What a lane needs at the ends of its queries only, and its ray as the tests read it.
+struct LaneShared {
+    float4 o[32], s[32];                 // as grid_tri_test takes them
+    float ox[32], oy[32], oz[32], dx[32], dy[32], dz[32];
+    float E[32], gE[32], lam[32], mu[32], d_int[32];
+    int crossed[32], may_cross[32];      // crossings applied; segments left to the cap
+    int where[32];                       // region | instance << 8
+    unsigned int qidx[32];
+};
+template <bool GRAD, bool COUNT>
+__global__ void __launch_bounds__(256, 4) trace_grid_kernel(const Params P, State S, int cur,
+                                                             unsigned long long *counters)
+{
+    const uint32_t FULL = 0xffffffffu;
+    const GridSet &G = P.grid;
+    extern __shared__ int4 s_reg[];
+    __shared__ LaneShared s_lane[8];
+    for (int i = threadIdx.x; i < P.n_region; i += blockDim.x) s_reg[i] = P.regions[i];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    LaneShared &L = s_lane[threadIdx.x >> 5];
+    const unsigned int n = S.ctrl->q_count[cur];
+    const unsigned int *queue = S.qsort;
+    bool has = false, reloc = false;
+    int word = 0;                                // of the walk's cell; 0 = the query is done
+    uint32_t li = 0, ln = 0;                     // list of the cell: next entry, tests left
+    int next = 0, exclude = -1;                  // triangle of the next test
+    Walk w{};
+    Nearest h{ 0.0f, 0.0f, 1.0f, -1 };
+    uint32_t lists = 0;
+    uint32_t nn = 0, nt = 0;
+    // warp-uniform private range [wb, we) of the queue, refilled a chunk at a time
+    unsigned int wb = 0, we = 0;
+    bool global_done = false, drained = false;
+    auto open_cell = [&]() {
+        if (word < 0) {
+            li = cell_list(G.list, lists, word, ln);
+            next = (int)__ldg(G.list + li);
+            word = __float_as_int(1.0f);         // once its tests are done, the cell alone is left
+        }
+    };
+    while (true) {
+        uint32_t m_test = __ballot_sync(FULL, ln != 0);
+        uint32_t m_step = __ballot_sync(FULL, word != 0 && ln == 0);
+        const uint32_t m_done = __ballot_sync(FULL, has && word == 0);
+        const int n_test = __popc(m_test), n_step = __popc(m_step);
+        const int n_idle = drained ? 0 : __popc(~(m_step | m_test | m_done));
+        const bool serve = __popc(m_done) + n_idle >= kServeMin || !(m_test | m_step);
+        if (n_test >= kTestMin || (n_test > n_step && !serve)) {
+            // ---- triangle tests, one per lane and pass ----
+            do {
+                if (ln) {
+                    const int id = next;
+                    if (--ln) next = (int)__ldg(G.list + ++li);
+                    if (COUNT) ++nt;
+                    const float4 o = L.o[lane], s = L.s[lane];
+                    float num, den;
+                    if (grid_tri_test(G, o, s, id, num, den) && id != exclude)
+                        nearer(h, num, den, id, __float_as_int(s.w) < 0, o.w);
+                }
+                m_test = __ballot_sync(FULL, ln != 0);
+            } while (__popc(m_test) >= kTestMin);
+            continue;
+        }
+        if (n_step >= kStepMin || (m_step && !serve)) {
+            // ---- steps from cell to cell ----
+            do {
+                if (word != 0 && ln == 0) {
+                    if (COUNT) ++nn;
+                    word = walk_step(w, __int_as_float(word)) >= h.t ? 0 : walk_word(w, G.cells);
+                    open_cell();
+                }
+                m_step = __ballot_sync(FULL, word != 0 && ln == 0);
+            } while (__popc(m_step) >= kStepMin);
+            continue;
+        }
+        if (!m_done && !n_idle) break;           // nothing is left: serve is set by m_test | m_step == 0
+        bool begin = false;
+        // ---- queries that are done: cross, relocate, or store the hit ----
+        if (has && word == 0) {
+            const int where = L.where[lane], region = where & 255;
+            const bool left_out = h.best >= 0 && (h.best & kTied) != 0;     // the tree's to answer
+            const int best = left_out ? -1 : h.best >> 1;
+            const bool ent = (h.best & 1) != 0, bounded = L.d_int[lane] < INFINITY;
+            const float t_min = L.o[lane].w;
+            float t_hit = INFINITY;
+            int treg = 0;
+            if (best >= 0) {
+                t_hit = nearest_t(P.planes, h, L.ox[lane], L.oy[lane], L.oz[lane], L.dx[lane], L.dy[lane], L.dz[lane],
+                                  t_min);
+                treg = __float_as_int(__ldg(&G.tris[3 * best].w));
+                const float len = t_hit - t_min;
+                const float left = fmaf(-L.mu[lane], len, L.lam[lane]);
+                if (!reloc && !(L.d_int[lane] < len) && L.crossed[lane] < L.may_cross[lane] && isfinite(left)) {
+                    if (GRAD) {
+                        const int group = (s_reg[region].y >> 1) - 1;
+                        if (group >= 0 && group < 4) {
+                            float pe = 0.0f, co = 0.0f, pa = 0.0f;
+                            if (s_reg[region].x >= 0)
+                                mu_on_grid(P.xs + (size_t)s_reg[region].x * P.n_grid, P.n_grid, L.gE[lane], L.E[lane], pe,
+                                           co, pa);
+                            float *sc = reinterpret_cast<float *>(&S.score[queue[L.qidx[lane]]]) + group;
+                            *sc = fmaf(-(pe + co + pa), len, *sc);
+                        }
+                    }
+                    L.lam[lane] = left;
+                    L.o[lane].w = t_hit;
+                    exclude = best;
+                    L.where[lane] = (where & ~255) | (ent ? treg : s_reg[treg].z);
+                    ++L.crossed[lane];
+                    begin = true;
+                }
+            } else if (!left_out && !bounded && region != 0 && !reloc) {
+                // Inside a solid every ray meets the solid's boundary, so a photon whose
+                // region has no surface ahead sits a rounding error past it (an
+                // interaction point computed in FP32 right at a surface): search every
+                // triangle instead; physics then takes the photon to the region of the
+                // surface found, or to the world when there is none.
+                reloc = true;
+                begin = true;
+            }
+            if (!begin) {
+                const unsigned int qidx = L.qidx[lane];
+                const int crossed = L.crossed[lane];
+                Hit ht;
+                ht.tri = best;
+                ht.t = t_hit;
+                ht.region = treg;
+                ht.code = kCodeBias + (best >= 0 ? (ent ? 1 : 0) + (reloc ? kRelocated : 0)
+                                                 : (reloc ? kRelocated : (bounded ? kBeyond : 0)));
+                if (left_out) S.left[atomicAdd(&S.ctrl->n_left, 1u)] = qidx;
+                ht.code |= crossed << kCodeBits;
+                S.hit[qidx] = ht;
+                if (crossed)
+                    S.hot[qidx].f = make_float4(t_min, __uint_as_float(ray_tag(exclude, region)), L.E[lane], L.lam[lane]);
+                has = false;
+                reloc = false;
+            }
+        }
+        // ---- dynamic fetch: lanes without a ray take the next queue entries ----
+        const uint32_t need = __ballot_sync(FULL, !has);
+        if (!drained && (__popc(need) >= kFetchMin || !__ballot_sync(FULL, word != 0 || begin))) {
+            const unsigned int k = __popc(need);
+            const unsigned int avail = we - wb;
+            unsigned int nb = 0, ne = 0;
+            if (avail < k && !global_done) {
+                if (lane == 0) nb = atomicAdd(&S.ctrl->trace_head, (unsigned int)kTraceChunk);
+                nb = __shfl_sync(FULL, nb, 0);
+                if (nb >= n) { global_done = true; nb = ne = n; }
+                else ne = min(nb + (unsigned int)kTraceChunk, n);
+            }
+            const unsigned int rank = __popc(need & ((1u << lane) - 1u));
+            unsigned int idx = 0xffffffffu;
+            if (rank < avail) idx = wb + rank;
+            else if (nb + (rank - avail) < ne) idx = nb + (rank - avail);
+            if (avail >= k) wb += k;
+            else if (ne > nb) { wb = min(nb + (k - avail), ne); we = ne; }
+            else wb = we;
+            drained = global_done && wb >= we;
+            if (!has && idx != 0xffffffffu) {
+                L.qidx[lane] = idx;
+                const Slot &sr = S.slot[queue[idx]];
+                const SlotA sa = sr.a;
+                S.hot[idx] = sa;        // physics reads it here, in queue order
+                const float4 af = sa.f;
+                const float4 bo = sr.b.o, bd = sr.b.d;
+                L.E[lane] = af.z;
+                L.gE[lane] = (logf(af.z) - P.lnE_min) * P.inv_dlnE;
+                L.lam[lane] = af.w;
+                const uint32_t tag = __float_as_uint(af.y);
+                L.ox[lane] = bo.x; L.oy[lane] = bo.y; L.oz[lane] = bo.z;
+                exclude = (int)(tag >> kTagShift) - 1;
+                L.where[lane] = (int)((tag & 255u) | (sa.u.x & kInstMask) << 8);
+                const GridRay r = grid_ray(G, make_shear_k(bd.x, bd.y, bd.z), bo.x, bo.y, bo.z);
+                L.o[lane] = make_float4(r.ox, r.oy, r.oz, af.x);
+                L.s[lane] = make_float4(r.sx, r.sy, r.sz, __uint_as_float((uint32_t)(r.tris - G.tris) |
+                                                                         (r.flip ? 0x80000000u : 0u)));
+                L.dx[lane] = back_from_reciprocal(bd.x);
+                L.dy[lane] = back_from_reciprocal(bd.y);
+                L.dz[lane] = back_from_reciprocal(bd.z);
+                L.crossed[lane] = 0;
+                int may = (int)min((uint32_t)P.step_cap - min(sa.u.y, (uint32_t)P.step_cap), (uint32_t)kMaxCrossed);
+                if ((sa.u.x >> kErrShift) & kErrMask) may = 0;    // ends at its next physics visit
+                L.may_cross[lane] = may;
+                has = true;
+                begin = true;
+            }
+        }
+        // ---- the next segment of the lanes that crossed or fetched ----
+        if (begin) {
+            const int where = L.where[lane], region = where & 255;
+            float d_int = INFINITY;
+            if (!reloc) {
+                const int4 reg = s_reg[region];
+                float mu = 0.0f;
+                if (reg.x >= 0) {
+                    float pe, co, pa;
+                    mu_on_grid(P.xs + (size_t)reg.x * P.n_grid, P.n_grid, L.gE[lane], L.E[lane], pe, co, pa);
+                    const int group = (reg.y >> 1) - 1;
+                    const float scl = group >= 0 ? __ldg(&P.inst[where >> 8].scale[group]) : 1.0f;
+                    mu = (pe + co + pa) * scl;
+                    if (mu > 0.0f) d_int = L.lam[lane] / mu;
+                }
+                L.mu[lane] = mu;
+                L.d_int[lane] = d_int;
+            }
+            const float t_min = L.o[lane].w;
+            h.t = h.num = fmaf(d_int, 1.0f + 1.0f / 1024.0f, t_min) + 1e-3f;
+            h.den = 1.0f;
+            h.best = -1;
+            word = walk_begin(w, G, reloc ? G.all : region, L.ox[lane], L.oy[lane], L.oz[lane], L.dx[lane], L.dy[lane],
+                              L.dz[lane], t_min, lists);
+            open_cell();
+        }
+    }
+    if (COUNT) {
+        atomicAdd(&counters[0], (unsigned long long)nn);
+        atomicAdd(&counters[1], (unsigned long long)nt);
+        atomicAdd(&counters[3], (unsigned long long)nn);
+    }
+}
+
+// traverse() out of line, for the few queries that the grids leave to the tree
+// (entering -2: its stack overflowed).
+struct TreeHit { float t; int tri, entering; };
+static __device__ __noinline__ TreeHit tree_nearest(const float4 *nodes, const float4 *slots, const float4 *planes,
+                                                    int root, float ox, float oy, float oz, float dx, float dy,
+                                                    float dz, float t_min, int exclude, float t_max)
+{
+    float t = INFINITY;
+    bool entering = false;
+    uint32_t err = 0;
+    TravStats st{};
+    const int hit = traverse<false>(nodes, slots, planes, root, ox, oy, oz, dx, dy, dz, t_min, exclude, t, entering, err,
+                                    st, t_max);
+    return TreeHit{ t, hit >= 0 ? __float_as_int(__ldg(&slots[3 * hit + 1].w)) : -1,
+                    (err & ERR_STACK) ? -2 : (entering ? 1 : 0) };
+}
+
+// The queries that trace_grid_kernel left to the tree (two triangles at one distance:
+// about one query in 10^7), one per thread, at the segment where it left them.
+__global__ void __launch_bounds__(128) left_kernel(const Params P, State S)
+{
+    const unsigned int n = S.ctrl->n_left;
+    for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned int qidx = S.left[i];
+        const SlotA a = S.hot[qidx];
+        const SlotB b = S.slot[S.qsort[qidx]].b;
+        const float t_min = a.f.x;
+        const uint32_t tag = __float_as_uint(a.f.y);
+        const int4 R = P.regions[tag & 255u];
+        float t_max = INFINITY;
+        if (R.x >= 0) {
+            float pe, co, pa;
+            mu_at(P.xs + (size_t)R.x * P.n_grid, P.n_grid, P.lnE_min, P.inv_dlnE, a.f.z, pe, co, pa);
+            const int group = (R.y >> 1) - 1;
+            const float mu = (pe + co + pa) * (group >= 0 ? P.inst[a.u.x & kInstMask].scale[group] : 1.0f);
+            if (mu > 0.0f) t_max = fmaf(a.f.w / mu, 1.0f + 1.0f / 1024.0f, t_min) + 1e-3f;
+        }
+        const int exclude = (int)(tag >> kTagShift) - 1;
+        bool reloc = false;
+        TreeHit k = tree_nearest(P.nodes, P.tris, P.planes, R.w, b.o.x, b.o.y, b.o.z, b.d.x, b.d.y, b.d.z, t_min, exclude,
+                                 t_max);
+        if (k.tri < 0 && k.entering != -2 && !(t_max < INFINITY) && (tag & 255u) != 0u) {
+            reloc = true;
+            k = tree_nearest(P.nodes, P.tris, P.planes, P.root_all, b.o.x, b.o.y, b.o.z, b.d.x, b.d.y, b.d.z, t_min,
+                             exclude, t_max);
+        }
+        Hit h = S.hit[qidx];
+        h.t = k.t;
+        h.tri = k.tri;
+        h.region = k.tri >= 0 ? __float_as_int(__ldg(&P.grid.tris[3 * k.tri].w)) : 0;
+        h.code = (h.code & ~((1 << kCodeBits) - 1)) |
+                 (kCodeBias + (k.entering == -2 ? -2
+                               : k.tri >= 0 ? k.entering + (reloc ? kRelocated : 0)
+                                            : (reloc ? kRelocated : (t_max < INFINITY ? kBeyond : 0))));
+        S.hit[qidx] = h;
+    }
+}
+
 // ---------------------------------------------------------------- physics
 // Bounds on registers: with room for three blocks of 256 per SM, ptxas allocates the
 // photon-only form without spilling in 64 registers (so four blocks still fit; under a
 // four-block bound it spilled a few bytes and ran slower) and the charged-particle form
 // in 80; the gradient form would take 69 and drop to three blocks per SM, slower than
 // its small spill at four, so it keeps the four-block bound.
-template <bool GRAD, bool COUNT, bool EM>
+template <bool GRAD, bool COUNT, bool EM, bool GRID>
 __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params P, State S, int cur,
                                                       unsigned long long *counters)
 {
@@ -936,7 +1238,8 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
             const uint32_t info = sa.u.x;
             inst = (int)(info & kInstMask);
             uint32_t herr = (info >> kErrShift) & kErrMask, flags = (info >> kFlagShift) & kFlagMask;
-            uint32_t cell = info >> kCellShift, steps = sa.u.y;
+            const int hcode = (ht.code & ((1 << kCodeBits) - 1)) - kCodeBias;
+            uint32_t cell = info >> kCellShift, steps = sa.u.y + (uint32_t)(ht.code >> kCodeBits);
             int region = (int)(tag & 255u);
             int last_tri = (int)(tag >> kTagShift) - 1;
             const float4 sc4 = GRAD ? S.score[slot] : make_float4(0, 0, 0, 0);
@@ -963,15 +1266,15 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
                 inter_acc = 0;
                 inter_inst = inst;
             }
-            if (ht.entering == -2) herr |= ERR_STACK;
+            if (hcode == -2) herr |= ERR_STACK;
             if (++steps > (uint32_t)P.step_cap) herr |= ERR_STEPCAP;
             if (herr) {
                 finished = true;
             } else {
                 const float t_hit = ht.t;
                 const int hit_tri = ht.tri, hit_region = ht.region;
-                const bool entering = ht.entering == 1 || ht.entering == 1 + kRelocated;
-                if (ht.entering >= kRelocated) {
+                const bool entering = hcode == 1 || hcode == 1 + kRelocated;
+                if (hcode >= kRelocated) {
                     // the trace kernel relocated the photon (a rounding error past a
                     // boundary) by the nearest surface of the whole mesh; with none
                     // ahead it is outside every solid
@@ -1073,7 +1376,7 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
                             tr.tag = (uint32_t)region | ((uint32_t)inst << 8);
                         } else {
                             float e_esc = 0.0f;
-                            e_track<COUNT, false>(P, s_reg, I.scale, px, py, pz, eux, euy, euz, eT, ew, region, edep,
+                            e_track<COUNT, GRID>(P, s_reg, I.scale, px, py, pz, eux, euy, euz, eT, ew, region, edep,
                                            dep_all, e_esc, herr, ts);
                             esc_now += e_esc;
                         }
@@ -1217,7 +1520,7 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
 // The charged-particle tracks physics deferred in this iteration (e_model 1), one
 // per thread: their deposits and escapes join the history in its slot, and an
 // error of the track becomes the history's, before the slot's next physics visit.
-template <bool COUNT>
+template <bool COUNT, bool GRID>
 __global__ void __launch_bounds__(256) etrack_kernel(const Params P, State S, unsigned long long *counters)
 {
     __shared__ int4 s_reg[256];
@@ -1230,7 +1533,7 @@ __global__ void __launch_bounds__(256) etrack_kernel(const Params P, State S, un
         const int region = (int)(t.tag & 255u), inst = (int)(t.tag >> 8);
         float edep = 0.0f, dep_all = 0.0f, esc = 0.0f;
         uint32_t herr = 0;
-        e_track<COUNT, false>(P, s_reg, P.inst[inst].scale, t.p.x, t.p.y, t.p.z, t.u.x, t.u.y, t.u.z, t.p.w, t.u.w, region,
+        e_track<COUNT, GRID>(P, s_reg, P.inst[inst].scale, t.p.x, t.p.y, t.p.z, t.u.x, t.u.y, t.u.z, t.p.w, t.u.w, region,
                        edep, dep_all, esc, herr, ts);
         SlotA &a = S.slot[t.slot].a;
         uint4 u = a.u;
@@ -1313,6 +1616,7 @@ gadep_status wavefront_create(int device, int slots, bool grad, WavefrontBuffers
     size_t o_d0 = off; off = align_up(off + n * 4);
     size_t o_pend = off; off = align_up(off + ring * sizeof(unsigned long long));
     size_t o_ctrl = off; off = align_up(off + sizeof(wf::Ctrl));
+    size_t o_left = off; off = align_up(off + n * 4);
     size_t o_qlog = off; off = align_up(off + sizeof(unsigned int) * wf::kQueueLog);
     cudaError_t e = cudaMalloc(&w->block, off);
     if (e != cudaSuccess) {
@@ -1347,6 +1651,7 @@ gadep_status wavefront_create(int device, int slots, bool grad, WavefrontBuffers
     w->S.pend_mask = ring - 1;
     w->S.gen_target = target;
     w->S.ctrl = (wf::Ctrl *)(b + o_ctrl);
+    w->S.left = (unsigned int *)(b + o_left);
     w->S.qlog = (unsigned int *)(b + o_qlog);
     w->S.slots = slots;
     *out = w;
@@ -1362,6 +1667,20 @@ void wavefront_destroy(WavefrontBuffers *w)
     cudaFree(w->block);
     cudaFreeHost(w->host_ctrl);
     delete w;
+}
+
+// GRID matters to the charged-particle form alone: the others trace nothing.
+static const void *physics_of(bool grad, bool count, bool em, bool grid)
+{
+    using namespace wf;
+    if (grad) return count ? (const void *)physics_kernel<true, true, false, false>
+                           : (const void *)physics_kernel<true, false, false, false>;
+    if (!em) return count ? (const void *)physics_kernel<false, true, false, false>
+                          : (const void *)physics_kernel<false, false, false, false>;
+    if (grid) return count ? (const void *)physics_kernel<false, true, true, true>
+                           : (const void *)physics_kernel<false, false, true, true>;
+    return count ? (const void *)physics_kernel<false, true, true, false>
+                 : (const void *)physics_kernel<false, false, true, false>;
 }
 
 // Run every history of the plan's Params through the wavefront kernels on `s`.
@@ -1405,12 +1724,7 @@ gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P0, bool grad
         };
         set((const void *)wf::gen_kernel, gsm);
         set((const void *)wf::sort_kernel, ssm);
-        set((const void *)wf::physics_kernel<true, true, false>, rsm);
-        set((const void *)wf::physics_kernel<true, false, false>, rsm);
-        set((const void *)wf::physics_kernel<false, true, false>, rsm);
-        set((const void *)wf::physics_kernel<false, false, false>, rsm);
-        set((const void *)wf::physics_kernel<false, true, true>, rsm);
-        set((const void *)wf::physics_kernel<false, false, true>, rsm);
+        set(physics_of(grad, count, P.e_model != 0, P.grid.desc != nullptr), rsm);
         if (e != cudaSuccess) return fail(GADEP_E_CUDA, "wavefront: shared memory: %s", cudaGetErrorString(e));
     }
     const unsigned long long max_iter = (unsigned long long)P.step_cap * 4 + P.total / 1024 + 1000000ull;
@@ -1438,21 +1752,27 @@ gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P0, bool grad
             args[0] = &S; args[1] = &c; args[2] = (void *)&n_keys; break;
         case KK_N: fn = (const void *)wf::sort_prefix_kernel; block = dim3(1024);   // the sort's prefix
             args[0] = &S; args[1] = &c; args[2] = (void *)&n_keys; break;
-        case KK_TRACE: fn = count ? (const void *)wf::trace_kernel<true> : (const void *)wf::trace_kernel<false>;
-            grid = dim3(w->trace_grid);
-            args[0] = &P; args[1] = &S; args[2] = &c; args[3] = &counters; break;
-        case KK_PHYSICS:
-            if (grad)
-                fn = count ? (const void *)wf::physics_kernel<true, true, false>
-                           : (const void *)wf::physics_kernel<true, false, false>;
-            else if (P.e_model)
-                fn = count ? (const void *)wf::physics_kernel<false, true, true>
-                           : (const void *)wf::physics_kernel<false, false, true>;
+        case KK_TRACE:
+            if (P.grid.desc)
+                fn = grad ? (count ? (const void *)wf::trace_grid_kernel<true, true>
+                                   : (const void *)wf::trace_grid_kernel<true, false>)
+                          : (count ? (const void *)wf::trace_grid_kernel<false, true>
+                                   : (const void *)wf::trace_grid_kernel<false, false>);
             else
-                fn = count ? (const void *)wf::physics_kernel<false, true, false>
-                           : (const void *)wf::physics_kernel<false, false, false>;
+                fn = count ? (const void *)wf::trace_kernel<true> : (const void *)wf::trace_kernel<false>;
+            grid = dim3(w->trace_grid);
+            smem = P.grid.desc ? (size_t)P.n_region * sizeof(int4) : 0;
+            args[0] = &P; args[1] = &S; args[2] = &c; args[3] = &counters; break;
+        case KK_N + 5: fn = (const void *)wf::left_kernel; block = dim3(128);
+            args[0] = &P; args[1] = &S; break;
+        case KK_PHYSICS:
+            fn = physics_of(grad, count, P.e_model != 0, P.grid.desc != nullptr);
             grid = dim3(w->work_grid); smem = rsm; args[0] = &P; args[1] = &S; args[2] = &c; args[3] = &counters; break;
-        case KK_ETRACK: fn = count ? (const void *)wf::etrack_kernel<true> : (const void *)wf::etrack_kernel<false>;
+        case KK_ETRACK:
+            if (P.grid.desc)
+                fn = count ? (const void *)wf::etrack_kernel<true, true> : (const void *)wf::etrack_kernel<false, true>;
+            else
+                fn = count ? (const void *)wf::etrack_kernel<true, false> : (const void *)wf::etrack_kernel<false, false>;
             grid = dim3(w->work_grid); args[0] = &P; args[1] = &S; args[2] = &counters; break;
         default: return cudaErrorInvalidValue;
         }
@@ -1468,14 +1788,13 @@ gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P0, bool grad
     };
     // the kernels of one iteration; the deferred charged-particle tracks run right
     // after physics
-    int kIteration[8] = { KK_SPAWN, KK_N, KK_SORT, KK_TRACE, KK_PHYSICS, KK_GEN, KK_CTRL, KK_CTRL };
-    int n_iter = 7;
-    if (P.e_model) {
-        kIteration[5] = KK_ETRACK;
-        kIteration[6] = KK_GEN;
-        kIteration[7] = KK_CTRL;
-        n_iter = 8;
-    }
+    int kIteration[10], n_iter = 0;
+    for (int k : { (int)KK_SPAWN, (int)KK_N, (int)KK_SORT, (int)KK_TRACE }) kIteration[n_iter++] = k;
+    if (P.grid.desc) kIteration[n_iter++] = KK_N + 5;          // the queries left; timed with the trace
+    kIteration[n_iter++] = KK_PHYSICS;
+    if (P.e_model) kIteration[n_iter++] = KK_ETRACK;
+    kIteration[n_iter++] = KK_GEN;
+    kIteration[n_iter++] = KK_CTRL;
     KernelTimer none;
     KernelTimer &T = timer ? *timer : none;
 
@@ -1566,9 +1885,10 @@ gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P0, bool grad
         const int cur = (int)(it & 1);
         for (int k = 0; k < n_iter; ++k) {
             const int kind = kIteration[k];
-            if (kind != KK_SORT) T.before(s);      // the prefix and the sort are timed together
+            // the prefix and the sort are timed together, and the trace and the queries it left
+            if (kind != KK_SORT && kind <= KK_N) T.before(s);
             const cudaError_t e = launch(kind, cur, nullptr, nullptr, 0, nullptr, 0, 0);
-            if (kind != KK_N) T.after(kind, s);
+            if (kind != KK_N && !(kind == KK_TRACE && P.grid.desc)) T.after(kind > KK_N ? KK_TRACE : kind, s);
             if (e != cudaSuccess) return fail(GADEP_E_CUDA, "wavefront: launch: %s", cudaGetErrorString(e));
         }
         if (it % check_every == check_every - 1) {
