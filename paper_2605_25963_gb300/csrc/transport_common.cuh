@@ -394,9 +394,11 @@ dev::GridSet grid_set(const gadep_bvh *b);
 gadep_status wavefront_create(int device, int slots, bool grad, WavefrontBuffers **out);
 void wavefront_destroy(WavefrontBuffers *w);
 // slots: photon slots the run keeps in flight (at most the buffers' capacity; 0 =
-// the capacity).
+// the capacity).  sort_births: the first births take their slots in the order of their
+// directions.
 gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P, bool grad, bool count,
-                           unsigned long long *counters, KernelTimer *timer, cudaStream_t s, int slots);
+                           unsigned long long *counters, KernelTimer *timer, cudaStream_t s, int slots,
+                           bool sort_births);
 int wavefront_trace_grid(const WavefrontBuffers *w);
 gadep_status wavefront_check(WavefrontBuffers *w, cudaStream_t s);
 gadep_status wavefront_queue_log(WavefrontBuffers *w, uint32_t *out, int max, int *n, cudaStream_t s);
