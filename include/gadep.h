@@ -309,7 +309,7 @@ typedef struct {
                                  expected to reach the scene (the mesh's bounding box), else the
                                  megakernel */
     int32_t  block;           /* threads per block (0 = default) */
-    int32_t  chunk;           /* histories a warp takes from the work counter at once (0 = default) */
+    int32_t  chunk;           /* histories a warp takes from the work counter at once (0 = by what is left) */
     int32_t  blocks_per_sm;   /* persistent grid = SMs x this (0 = occupancy maximum) */
     int32_t  n_group;         /* density groups scored by gadep_grad (<= 4) */
     float    group_scale[GADEP_MAX_GROUPS];  /* density scale per group (default 1) */

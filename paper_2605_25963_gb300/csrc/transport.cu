@@ -1,7 +1,7 @@
 // transport.cu -- GPU photon transport through the detector mesh (paper Sec. 2.4).
 //
 // One persistent "megakernel" runs whole histories.  Every warp takes histories
-// from a device work counter in chunks (the work queue of a batched run is the
+// from a device work counter in chunks (set_chunk; the work queue of a batched run is the
 // flattened history range of all instances, so one launch serves any number of
 // instances with uneven history counts); a lane whose history ends takes the
 // next one at once, so lanes stay busy while long histories continue.
@@ -50,6 +50,7 @@ namespace dev {
 // EM: charged-particle tracks (e_model 1), a separate instantiation so that the
 // photon-only kernels keep their registers.  GRID: the queries walk the regions'
 // grids (grid.cuh) instead of their trees.
+constexpr int kMaxChunk = 256;
 template <bool GRAD, bool COUNT, bool EM, bool GRID>
 // 4 blocks of 256 threads per SM (64 registers): measured faster than 2 or 3
 // blocks despite the register spills, as the traversal is latency bound.
@@ -96,12 +97,15 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
         uint32_t need = __ballot_sync(FULL, !busy);
         while (need && !exhausted) {
             if (pool_next == pool_end) {
+                // a share of what the warp knows to be left, in whole warps
+                const int share = (int)((float)(P.total - pool_end) * P.share) & ~31;
+                const unsigned long long chunk = (unsigned long long)max(P.chunk, min(share, kMaxChunk));
                 unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(P.work, (unsigned long long)P.chunk);
+                if (lane == 0) base = atomicAdd(P.work, chunk);
                 base = __shfl_sync(FULL, base, 0);
                 if (base >= P.total) { exhausted = true; break; }
                 pool_next = base;
-                pool_end = min(base + (unsigned long long)P.chunk, P.total);
+                pool_end = min(base + chunk, P.total);
             }
             const uint32_t avail = (uint32_t)(pool_end - pool_next);
             const uint32_t take = min((uint32_t)__popc(need), avail);
@@ -840,6 +844,20 @@ dev::GridSet grid_of(const gadep_bvh *b, const dev::InstDev *inst, int n_inst, i
     return g;
 }
 
+// The megakernel's histories come to its warps in chunks.  Of what is left a warp takes half
+// its share, at most 256 and at least the 32 that fill it once: large chunks spare the work
+// counter while there is much to do, small ones keep every warp busy in short runs and at the
+// end of long ones.  With 256 at any time 20,000 histories were the work of 79 warps out of
+// 4,864.  Time of a run (256 at any time / now, us): coax 1e3 histories 682 / 334, 2e4 975 /
+// 384, 3e5 1152 / 636, 1e6 1506 / 1231; prism source 2e4 1816 / 533; bare cylinder 2e4 182 /
+// 160, 1e6 275 / 275; detector 2 at 250 mm, 1e7 929 / 913.  A quarter, eighth or sixteenth of
+// a share: within 2 % of a half, and 960 in the last case.
+void set_chunk(dev::Params &P, const gadep_opts *opts, int n_warps)
+{
+    P.chunk = opts->chunk > 0 ? opts->chunk : 32;
+    P.share = opts->chunk > 0 ? 0.0f : 1.0f / (float)(2 * n_warps);
+}
+
 gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t n_inst,
                          const gadep_instance *inst, const gadep_opts *opts, bool grad, bool count,
                          gadep_plan **out)
@@ -1158,7 +1176,7 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
     P.n_bins = opts->n_bins;
     P.step_cap = opts->step_cap;
     P.n_group = opts->n_group;
-    P.chunk = opts->chunk > 0 ? opts->chunk : 256;
+    set_chunk(P, opts, p->grid * (p->block / 32));
     P.n_stripes = p->n_stripes;
     P.root_all = b->root_all;
     P.erange = p->d_erange;
@@ -1696,7 +1714,7 @@ extern "C" gadep_status gadep_run_noalloc(const gadep_bvh *b, const gadep_materi
     P.n_bins = opts->n_bins;
     P.step_cap = opts->step_cap;
     P.n_group = opts->n_group;
-    P.chunk = opts->chunk > 0 ? opts->chunk : 256;
+    set_chunk(P, opts, n_sm * bps * (block / 32));
     P.n_stripes = 1;                       // the one tally record of the scratch array
     P.root_all = b->root_all;
     gadep::scene_box(b, P.root_lo, P.root_hi);

@@ -51,7 +51,9 @@ struct Params {
     float lnE_min, inv_dlnE;
     uint32_t key0, key1;
     float e_cut, fep_delta, e_max, bin_scale;
-    int n_bins, step_cap, n_group, chunk;
+    int n_bins, step_cap, n_group;
+    int chunk;                    // megakernel: histories a warp takes at once, at least, and
+    float share;                  // the share of those left that it takes where that is more
     int n_stripes;                      // tally copies [n_stripes][n_inst], summed on the host
     float root_lo[3], root_hi[3];       // bounds of every triangle (padded)
     int root_all;                       // tree over every triangle
