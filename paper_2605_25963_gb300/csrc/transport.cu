@@ -50,8 +50,48 @@ namespace dev {
 // EM: charged-particle tracks (e_model 1), a separate instantiation so that the
 // photon-only kernels keep their registers.  GRID: the queries walk the regions'
 // grids (grid.cuh) instead of their trees.
+// Source point and direction of a history (the first words of its stream).
+__device__ __forceinline__ void birth(const InstDev &I, Stream &rng, uint32_t k0, uint32_t k1, float &ox, float &oy,
+                                      float &oz, float &dx, float &dy, float &dz)
+{
+    ox = I.px; oy = I.py; oz = I.pz;
+    if (I.src_kind == GADEP_SRC_DISK) {
+        const float r = I.radius * sqrtf(rng.u01(k0, k1));
+        float sp, cp;
+        sincospif(2.0f * rng.u01(k0, k1), &sp, &cp);
+        ox = fmaf(r, cp, ox); oy = fmaf(r, sp, oy);
+    } else if (I.src_kind == GADEP_SRC_PRISM) {
+        const int N = I.n_sides;
+        int kk = (int)((float)N * rng.u01(k0, k1));
+        kk = min(kk, N - 1);
+        const float s1 = sqrtf(rng.u01(k0, k1)), u3 = rng.u01(k0, k1);
+        float sa, ca, sb, cb;
+        sincospif(2.0f * (float)kk / (float)N, &sa, &ca);
+        sincospif(2.0f * (float)((kk + 1) % N) / (float)N, &sb, &cb);
+        const float wa = s1 * (1.0f - u3), wb = s1 * u3;
+        ox += I.radius * (wa * ca + wb * cb);
+        oy += I.radius * (wa * sa + wb * sb);
+        oz = fmaf(I.height, rng.u01(k0, k1), oz);
+    }
+    if (I.src_kind == GADEP_SRC_PENCIL) { dx = I.dx; dy = I.dy; dz = I.dz; }
+    else iso_dir(rng, k0, k1, dx, dy, dz);
+}
+
+// Whether history `local` of a source outside every solid starts towards the scene's box.
+// Out of line: the callers' photons keep their registers.
+static __device__ __noinline__ bool birth_reaches(const InstDev *I, unsigned long long local, uint32_t k0, uint32_t k1,
+                                                  float3 lo, float3 hi)
+{
+    Stream rng;
+    rng.init(I->hist_offset + local, I->inst_id);
+    float ox, oy, oz, dx, dy, dz;
+    birth(*I, rng, k0, k1, ox, oy, oz, dx, dy, dz);
+    const float l[3] = { lo.x, lo.y, lo.z }, h[3] = { hi.x, hi.y, hi.z };
+    return ray_hits_box(l, h, ox, oy, oz, dx, dy, dz);
+}
+
 constexpr int kMaxChunk = 256;
-template <bool GRAD, bool COUNT, bool EM, bool GRID>
+template <bool GRAD, bool COUNT, bool EM, bool GRID, bool SCAN>
 // 4 blocks of 256 threads per SM (64 registers): measured faster than 2 or 3
 // blocks despite the register spills, as the traversal is latency bound.
 __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsigned long long *counters)
@@ -73,7 +113,23 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
     const uint32_t k0 = P.key0, k1 = P.key1;
 
     unsigned long long pool_next = 0, pool_end = 0;
+    int pool_inst = 0;                  // instance of the histories at pool_next
+    uint32_t n_culled = 0;              // histories of it that ended at birth, not yet tallied
     bool exhausted = false;
+    // histories found to reach the scene, in order, and not yet begun
+    constexpr uint32_t kFound = 64;
+    __shared__ unsigned long long s_found[SCAN ? 8 : 1][kFound];
+    unsigned long long *list = s_found[SCAN ? threadIdx.x >> 5 : 0];
+    uint32_t first = 0, found = 0;
+    auto cull = [&](int i, uint32_t n) {
+        if (lane != 0 || n == 0) return;
+        TallyDev &t = block_tally(P)[i];
+        atomicAdd(&t.n_hist, (unsigned long long)n);
+        atomicAdd(&t.n_zero, (unsigned long long)n);
+        atomicAdd(&t.n_segments, (unsigned long long)n);
+        atomicAdd(&t.n_culled, (unsigned long long)n);
+        atomicAdd(&t.sum_esc, (double)n * (double)P.inst[i].E0);
+    };
     bool busy = false;
     int inst = 0;
     unsigned long long g_hist = 0;
@@ -95,7 +151,74 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
     while (true) {
         // ---------------- refill idle lanes from the work counter ----------------
         uint32_t need = __ballot_sync(FULL, !busy);
-        while (need && !exhausted) {
+        while (SCAN && need) {
+            // Look for enough histories that reach the scene, all lanes together: each of
+            // the few idle ones by itself would test the 37 or 134 of a distant source that
+            // miss one after another, while the others wait.
+            while (found < (uint32_t)__popc(need) && found <= kFound - 32 && !exhausted) {
+                if (pool_next == pool_end) {
+                    // a share of what the warp knows to be left, in whole warps
+                    const int share = (int)((float)(P.total - pool_end) * P.share) & ~31;
+                    const unsigned long long chunk = (unsigned long long)max(P.chunk, min(share, kMaxChunk));
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(P.work, chunk);
+                    base = __shfl_sync(FULL, base, 0);
+                    if (base >= P.total) { exhausted = true; break; }
+                    pool_next = base;
+                    pool_end = min(base + chunk, P.total);
+                }
+                if (pool_next >= s_end[pool_inst]) {
+                    cull(pool_inst, n_culled);
+                    n_culled = 0;
+                    while (pool_next >= s_end[pool_inst]) ++pool_inst;
+                }
+                const InstDev *I = P.inst + pool_inst;
+                const uint32_t take = (uint32_t)min(min(pool_end, s_end[pool_inst]) - pool_next, 32ull);
+                const unsigned long long g = pool_next + lane;
+                bool reaches = lane < take;
+                if (reaches && I->birth_region == 0) {
+                    // Born in the world and aimed away from every solid: the one segment
+                    // of this history escapes with nothing deposited.
+                    reaches = birth_reaches(I, g - (pool_inst ? s_end[pool_inst - 1] : 0ull), k0, k1,
+                                            make_float3(P.root_lo[0], P.root_lo[1], P.root_lo[2]),
+                                            make_float3(P.root_hi[0], P.root_hi[1], P.root_hi[2]));
+                    if (!reaches && g < P.n_trace) P.edep_trace[g] = 0.0f;
+                }
+                const uint32_t m = __ballot_sync(FULL, reaches);
+                n_culled += take - __popc(m);
+                if (reaches) list[(first + found + __popc(m & lt_mask)) % kFound] = g;
+                found += __popc(m);
+                pool_next += take;
+            }
+            if (found == 0) break;
+            // The idle lanes begin those found, in order.
+            __syncwarp();
+            const uint32_t rank = __popc(need & lt_mask);
+            if (!busy && rank < found) {
+                g_hist = list[(first + rank) % kFound];
+                while (g_hist >= s_end[inst]) ++inst;
+                if (acc.inst != inst) { acc.flush_lane(block_tally(P)); acc.reset(inst); }
+                const InstDev &I = P.inst[inst];
+                rng.init(I.hist_offset + (g_hist - (inst ? s_end[inst - 1] : 0ull)), I.inst_id);
+                birth(I, rng, k0, k1, ox, oy, oz, dx, dy, dz);
+                E = E0 = I.E0;
+                region = I.birth_region;
+                t_cur = 0.0f; last_tri = -1; steps = 0;
+                has_sec = false;
+                edep = dep_all = esc = 0.0f;
+                herr = 0u;
+#pragma unroll
+                for (int g = 0; g < (GRAD ? 4 : 1); ++g) score[g] = 0.0f;
+                lam = -logf(rng.u01(k0, k1));
+                busy = true;
+            }
+            const uint32_t taken = min(found, (uint32_t)__popc(need));
+            first = (first + taken) % kFound;
+            found -= taken;
+            __syncwarp();
+            need = __ballot_sync(FULL, !busy);
+        }
+        while (!SCAN && need && !exhausted) {
             if (pool_next == pool_end) {
                 // a share of what the warp knows to be left, in whole warps
                 const int share = (int)((float)(P.total - pool_end) * P.share) & ~31;
@@ -117,27 +240,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                 const InstDev &I = P.inst[inst];
                 const unsigned long long local = g_hist - (inst ? s_end[inst - 1] : 0ull);
                 rng.init(I.hist_offset + local, I.inst_id);
-                ox = I.px; oy = I.py; oz = I.pz;
-                if (I.src_kind == GADEP_SRC_DISK) {
-                    const float r = I.radius * sqrtf(rng.u01(k0, k1));
-                    float sp, cp;
-                    sincospif(2.0f * rng.u01(k0, k1), &sp, &cp);
-                    ox = fmaf(r, cp, ox); oy = fmaf(r, sp, oy);
-                } else if (I.src_kind == GADEP_SRC_PRISM) {
-                    const int N = I.n_sides;
-                    int kk = (int)((float)N * rng.u01(k0, k1));
-                    kk = min(kk, N - 1);
-                    const float s1 = sqrtf(rng.u01(k0, k1)), u3 = rng.u01(k0, k1);
-                    float sa, ca, sb, cb;
-                    sincospif(2.0f * (float)kk / (float)N, &sa, &ca);
-                    sincospif(2.0f * (float)((kk + 1) % N) / (float)N, &sb, &cb);
-                    const float wa = s1 * (1.0f - u3), wb = s1 * u3;
-                    ox += I.radius * (wa * ca + wb * cb);
-                    oy += I.radius * (wa * sa + wb * sb);
-                    oz = fmaf(I.height, rng.u01(k0, k1), oz);
-                }
-                if (I.src_kind == GADEP_SRC_PENCIL) { dx = I.dx; dy = I.dy; dz = I.dz; }
-                else iso_dir(rng, k0, k1, dx, dy, dz);
+                birth(I, rng, k0, k1, ox, oy, oz, dx, dy, dz);
                 E = E0 = I.E0;
                 region = I.birth_region;
                 t_cur = 0.0f; last_tri = -1; steps = 0;
@@ -360,6 +463,9 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
             busy = false;
         }
     }
+    if (SCAN) cull(pool_inst, n_culled);
+    const int last = __reduce_max_sync(FULL, acc.inst);
+    if (acc.inst < 0) acc.inst = last;      // a lane that had no history: nothing to add
     flush_warp<GRAD>(acc, block_tally(P));
     if (COUNT) {
         atomicAdd(&counters[0], (unsigned long long)ts.nodes);
@@ -543,6 +649,7 @@ struct gadep_plan {
     int n_bins = 0;
     std::vector<gadep::dev::InstDev> inst;
     std::vector<unsigned long long> inst_end;
+    void *mega = nullptr;                    // the megakernel's form for this run
     void *scratch = nullptr;                 // one device block holding the buffers below
     bool scratch_cached = false;             // scratch borrowed from the BVH (with wf)
     float4 *d_xs = nullptr;
@@ -599,17 +706,31 @@ gadep_status check_opts(const gadep_opts *o)
 }
 
 template <bool GRID>
-void *kernel_of(bool grad, bool count, bool em)
+void *kernel_of(bool grad, bool count, bool em, bool scan)
 {
-    using namespace gadep::dev;
-    if (grad) return count ? (void *)transport_kernel<true, true, false, GRID> : (void *)transport_kernel<true, false, false, GRID>;
-    if (em) return count ? (void *)transport_kernel<false, true, true, GRID> : (void *)transport_kernel<false, false, true, GRID>;
-    return count ? (void *)transport_kernel<false, true, false, GRID> : (void *)transport_kernel<false, false, false, GRID>;
+    using gadep::dev::transport_kernel;
+    if (scan) return em ? (void *)transport_kernel<false, false, true, GRID, true> : (void *)transport_kernel<false, false, false, GRID, true>;
+    if (grad) return count ? (void *)transport_kernel<true, true, false, GRID, false> : (void *)transport_kernel<true, false, false, GRID, false>;
+    if (em) return count ? (void *)transport_kernel<false, true, true, GRID, false> : (void *)transport_kernel<false, false, true, GRID, false>;
+    return count ? (void *)transport_kernel<false, true, false, GRID, false> : (void *)transport_kernel<false, false, false, GRID, false>;
 }
 
-void *pick_kernel(bool grad, bool count, bool em, bool grid)
+void *pick_kernel(bool grad, bool count, bool em, bool grid, bool scan)
 {
-    return grid ? kernel_of<true>(grad, count, em) : kernel_of<false>(grad, count, em);
+    return grid ? kernel_of<true>(grad, count, em, scan) : kernel_of<false>(grad, count, em, scan);
+}
+
+// Whether a run's warps look for histories that reach the scene together: those of many
+// histories whose sources lie outside every solid.  Time of a run (lane by lane / together,
+// us): detector 2 at 250 mm, where 1 in 134 reaches it, 1e7 histories 927 / 878, 2e7 1844 /
+// 1158, 4e7 5758 / 2030; bare cylinder at 100 mm, 1 in 37, 1e6 270 / 270, 6e6 798 / 478; coax
+// at 25 mm, 1 in 4, 3e5 636 / 661, 1e6 1241 / 1134 (with charged-particle tracks 1771 / 1540).
+constexpr unsigned long long kScanMin = 3ull << 18;
+bool scans(bool grad, bool count, unsigned long long total, const gadep::dev::InstDev *inst, int n_inst)
+{
+    bool outside = total >= kScanMin && !grad && !count;
+    for (int i = 0; i < n_inst && outside; ++i) outside = inst[i].birth_region == 0;
+    return outside;
 }
 
 }  // namespace
@@ -983,7 +1104,9 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
         return fail(GADEP_E_INVAL, "plan: tables need %zu bytes of shared memory, the device has %d", smem, dev_smem);
     }
     p->P.grid = grid_of(b, p->inst.data(), n_inst, kMegaGridMinTri);
-    void *kfn = pick_kernel(grad, count, opts->e_model == 1, p->P.grid.desc != nullptr);
+    void *kfn = pick_kernel(grad, count, opts->e_model == 1, p->P.grid.desc != nullptr,
+                            scans(grad, count, total, p->inst.data(), n_inst));
+    p->mega = kfn;
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) { gadep_plan_destroy(p); return cuda_fail(e, "plan: cudaFuncSetAttribute"); }
     int bps = 0;
@@ -1212,8 +1335,7 @@ gadep_status plan_launch(gadep_plan *p, uint32_t *spectra_dev, float *edep_trace
     p->timer.before(s);
     {
         void *args[] = { &P, &p->d_counters };
-        e = cudaLaunchKernel(pick_kernel(p->grad, p->count, P.e_model != 0, P.grid.desc != nullptr), dim3(p->grid),
-                             dim3(p->block), args, (size_t)p->smem, s);
+        e = cudaLaunchKernel(p->mega, dim3(p->grid), dim3(p->block), args, (size_t)p->smem, s);
         if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "plan launch: kernel"); }
     }
     p->timer.after(KK_MEGA, s);
@@ -1665,7 +1787,7 @@ extern "C" gadep_status gadep_run_noalloc(const gadep_bvh *b, const gadep_materi
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, b->device);
     if (smem > (size_t)dev_smem) return fail(GADEP_E_INVAL, "gadep_run_noalloc: tables need too much shared memory");
     const dev::GridSet grid = grid_of(b, &d, 1, kMegaGridMinTri);
-    void *kfn = pick_kernel(false, false, false, grid.desc != nullptr);
+    void *kfn = pick_kernel(false, false, false, grid.desc != nullptr, scans(false, false, n_hist, &d, 1));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, block, smem);
     if (e == cudaSuccess && bps < 1) return fail(GADEP_E_CUDA, "gadep_run_noalloc: kernel does not fit on the device");
