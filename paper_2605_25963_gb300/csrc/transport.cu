@@ -4,7 +4,8 @@
 // from a device work counter in chunks (set_chunk; the work queue of a batched run is the
 // flattened history range of all instances, so one launch serves any number of
 // instances with uneven history counts); a lane whose history ends takes the
-// next one at once, so lanes stay busy while long histories continue.
+// next one at once, so lanes stay busy while long histories continue.  On larger
+// meshes its queries walk uniform grids (grid.cuh) instead of the trees.
 //
 // Per history (paper's Gadep step, photon part):
 //   birth        source position and isotropic direction (Philox stream of the

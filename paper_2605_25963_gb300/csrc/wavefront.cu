@@ -1,8 +1,9 @@
 // wavefront.cu -- wavefront form of the photon transport (same physics, same
 // Philox streams and same tallies as the persistent megakernel in transport.cu).
 //
-// Photons live in device-memory slots.  One iteration runs five kernels on the
-// stream, with no host round trip between them:
+// Photons live in device-memory slots.  One iteration runs these kernels on the
+// stream, with no host round trip between them (before the first, born_* put the births of
+// a large run with one source point in the order of their directions):
 //   spawn    free slots (popped from a stack) take births from the pending ring
 //            (an index map: the i-th popped slot gets the i-th pending history)
 //            and join the trace queue after the survivors of the previous iteration;
@@ -14,7 +15,8 @@
 //            the warp are still traversing (dynamic fetch), so the warp is not
 //            held by its longest ray; the hit is stored by queue position.  On
 //            middling meshes a second form walks uniform grids instead of the trees
-//            and applies the boundary crossings of a flight on the way;
+//            and applies the boundary crossings of a flight on the way, and a small
+//            kernel answers by the trees the few queries with two surfaces at one distance;
 //   physics  one thread per queued photon applies the segment: free flight,
 //            boundary crossing (nesting-tree rule), interaction or escape, and the
 //            end-of-history tally; survivors go to the next trace queue, finished
@@ -187,7 +189,8 @@ struct STally {
 template <bool GRAD>
 struct BlockTally {
     STally *t;
-    double *sc;                 // GRAD: [n_inst][8] fep score sums and squares
+    double *sc;                 // GRAD: [n_inst][kSums] fep score sums and squares, then the energies' sums
+    static constexpr int kSums = 11;
     int n;
     __device__ void init(void *smem, int n_inst)
     {
@@ -196,37 +199,24 @@ struct BlockTally {
         n = n_inst;
         for (int i = threadIdx.x; i < n_inst; i += blockDim.x) t[i] = STally{ 0, 0, 0, 0, 0, 0, 0, 0, 0.f, 0.f, 0.f, 0u };
         if (GRAD)
-            for (int i = threadIdx.x; i < 8 * n_inst; i += blockDim.x) sc[i] = 0.0;
+            for (int i = threadIdx.x; i < kSums * n_inst; i += blockDim.x) sc[i] = 0.0;
     }
-    __device__ void history(int inst, uint32_t segs, uint32_t herr, bool fep, float edep, float dep_all, float esc,
-                            float e_max, const float *score)
+    // GRAD: the scores of a history in the full-energy peak
+    __device__ void scores(int inst, const float *score)
     {
-        STally &s = t[inst];
-        atomicAdd(&s.hist, 1u);
-        atomicAdd(&s.seg, segs);
-        if (herr) {
-            atomicAdd(&s.err, 1u);
-            atomicOr(&s.errbits, herr);
-            return;
+        for (int g = 0; g < 4; ++g) {
+            const double v = (double)score[g];
+            atomicAdd(&sc[kSums * inst + g], v);
+            atomicAdd(&sc[kSums * inst + 4 + g], v * v);
         }
-        if (fep) {
-            atomicAdd(&s.fep, 1u);
-            if (GRAD)
-                for (int g = 0; g < 4; ++g) {
-                    const double v = (double)score[g];
-                    atomicAdd(&sc[8 * inst + g], v);
-                    atomicAdd(&sc[8 * inst + 4 + g], v * v);
-                }
-        }
-        if (edep == 0.0f) atomicAdd(&s.zero, 1u);
-        else if (edep >= e_max) atomicAdd(&s.over, 1u);
-        if (edep != 0.0f) atomicAdd(&s.dep, edep);
-        if (dep_all != 0.0f) atomicAdd(&s.dep_all, dep_all);
-        if (esc != 0.0f) atomicAdd(&s.esc, esc);
     }
     // The finished histories of a warp (every lane calls; fin: this lane finished
     // one): the lanes of one instance are summed in registers and one lane adds
     // the sums, instead of every lane adding its own.
+    // GRAD adds them in FP64: with crossings applied by the trace kernel more histories
+    // end in one launch, and FP32 block sums, a history at a time, put the deposits of
+    // runs of 6e6 histories 4.8e-9 off the FP64 value instead of 1.7e-9 (now 2.1e-9;
+    // physics of 1.2e7 histories 2.08 -> 1.99 ms, every lane adding in FP64 3.62).
     __device__ void history_warp(bool fin, int inst, uint32_t segs, uint32_t herr, bool fep, float edep,
                                  float dep_all, float esc, float e_max)
     {
@@ -261,9 +251,16 @@ struct BlockTally {
                 if (n_fep) atomicAdd(&s.fep, n_fep);
                 if (n_zero) atomicAdd(&s.zero, n_zero);
                 if (n_over) atomicAdd(&s.over, n_over);
-                if (d != 0.0f) atomicAdd(&s.dep, d);
-                if (da != 0.0f) atomicAdd(&s.dep_all, da);
-                if (e != 0.0f) atomicAdd(&s.esc, e);
+                if (GRAD) {
+                    double *sum = &sc[kSums * gi + 8];
+                    if (d != 0.0f) atomicAdd(&sum[0], (double)d);
+                    if (da != 0.0f) atomicAdd(&sum[1], (double)da);
+                    if (e != 0.0f) atomicAdd(&sum[2], (double)e);
+                } else {
+                    if (d != 0.0f) atomicAdd(&s.dep, d);
+                    if (da != 0.0f) atomicAdd(&s.dep_all, da);
+                    if (e != 0.0f) atomicAdd(&s.esc, e);
+                }
             }
         }
     }
@@ -293,13 +290,14 @@ struct BlockTally {
             if (s.seg) atomicAdd(&d.n_segments, (unsigned long long)s.seg);
             if (s.inter) atomicAdd(&d.n_interactions, (unsigned long long)s.inter);
             if (s.culled) atomicAdd(&d.n_culled, (unsigned long long)s.culled);
-            atomicAdd(&d.sum_dep_active, (double)s.dep);
-            atomicAdd(&d.sum_dep_all, (double)s.dep_all);
-            atomicAdd(&d.sum_esc, (double)s.esc);
+            const double *sum = GRAD ? &sc[kSums * i + 8] : nullptr;
+            atomicAdd(&d.sum_dep_active, GRAD ? sum[0] : (double)s.dep);
+            atomicAdd(&d.sum_dep_all, GRAD ? sum[1] : (double)s.dep_all);
+            atomicAdd(&d.sum_esc, GRAD ? sum[2] : (double)s.esc);
             if (GRAD)
                 for (int g = 0; g < 4; ++g) {
-                    atomicAdd(&d.fep_score[g], sc[8 * i + g]);
-                    atomicAdd(&d.fep_score_sq[g], sc[8 * i + 4 + g]);
+                    atomicAdd(&d.fep_score[g], sc[kSums * i + g]);
+                    atomicAdd(&d.fep_score_sq[g], sc[kSums * i + 4 + g]);
                 }
         }
     }
@@ -308,7 +306,7 @@ struct BlockTally {
 template <bool GRAD>
 __host__ __device__ constexpr size_t block_tally_bytes(int n_inst)
 {
-    return (size_t)n_inst * (sizeof(STally) + (GRAD ? 8 * sizeof(double) : 0));
+    return (size_t)n_inst * (sizeof(STally) + (GRAD ? BlockTally<true>::kSums * sizeof(double) : 0));
 }
 
 struct Ctrl {
@@ -995,8 +993,8 @@ __global__ void __launch_bounds__(256, 4) trace_kernel(const Params P, State S, 
 // between them: a photon that meets a surface before its interaction point goes on in
 // the region behind it at once, with physics' own arithmetic, so that physics sees a
 // photon once per flight and not once per segment.
-// Bound by instruction issue (70 % of issue slots, 16 of 32 lanes, L1 data pipe 71 %, DRAM
-// idle), so the warp's lanes are kept together: at any time the warp does the one thing
+// Bound by instruction issue (67 % of issue slots, 17 of 32 lanes, L1 data pipe 54 %, DRAM
+// 4 %), so the warp's lanes are kept together: at any time the warp does the one thing
 // that enough of its lanes wait for -- a step from cell to cell, a triangle test, or the
 // ends of queries and the fetch of new photons.  Lane by lane, without the votes, 8.8 of
 // 32 lanes had work (trace 34.2 ms per 1e8 histories at 1332 keV, 31.5 with them); tests
@@ -1560,11 +1558,8 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
                 float esc = 0.0f;
                 if (flags & kFlagEsc) esc = esc_now != 0.0f ? esc_now : S.esc[slot];
                 const bool fep = !herr && (I.E0 - edep) <= P.fep_delta;
-                if (GRAD) {
-                    bt.history(inst, steps, herr, fep, edep, dep_all, esc, P.e_max, score);
-                } else {
-                    fep_out = fep; dep_all_out = dep_all; esc_out = esc; segs_out = steps;
-                }
+                if (GRAD && fep) bt.scores(inst, score);
+                fep_out = fep; dep_all_out = dep_all; esc_out = esc; segs_out = steps;
                 if (P.n_trace) {
                     const uint32_t loc = have_b ? local : __float_as_uint(S.slot[slot].b.d.w);
                     const unsigned long long g = (inst ? P.inst_end[inst - 1] : 0ull) + loc;
@@ -1572,7 +1567,7 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
                 }
             }
         }
-        if (!GRAD) bt.history_warp(finished, inst, segs_out, herr_out, fep_out, edep_out, dep_all_out, esc_out, P.e_max);
+        bt.history_warp(finished, inst, segs_out, herr_out, fep_out, edep_out, dep_all_out, esc_out, P.e_max);
         // ---- spectrum atomics (warp-aggregated per bin) ----
         const bool binned = finished && herr_out == 0u && edep_out > 0.0f && edep_out < P.e_max;
         int bin = 0;
