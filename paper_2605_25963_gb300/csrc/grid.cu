@@ -25,7 +25,7 @@ constexpr double kGridPad = 0.02;           // of a cell, on every side
 constexpr double kCellsPerTri = 160.0;
 constexpr double kMinCells = 131072.0, kMaxCells = 4194304.0;  // per grid; indices stay below 2^23
 constexpr unsigned long long kMaxTotal = 1ull << 27;           // cells of all grids (2.4 GB while they are built)
-constexpr int kMinTris = 2048, kMaxTris = 1 << 18;      // no run walks the grids of other meshes
+constexpr int kMinTris = 2048, kMaxTris = 5 << 14;      // no run walks the grids of other meshes
 constexpr int kMaxSkip = 64;
 
 struct GridDesc {                           // host and build kernels

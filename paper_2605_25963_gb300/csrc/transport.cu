@@ -947,7 +947,10 @@ double hit_fraction(const dev::InstDev &d, const float lo[3], const float hi[3])
 // Meshes from this size on run the megakernel on the grids.  On the smallest the tree is a
 // few nodes: ms per run, tree / grids: 192 triangles 0.200 / 0.205, 3,456 triangles 0.81 /
 // 0.81, coax geometry 20,088 triangles 1e6 histories 2.13 / 1.41, 3e5 histories 1.12 /
-// 0.62, with charged-particle tracks 2.21 / 1.48, 216,684 triangles 2.36 / 2.14.
+// 0.62, with charged-particle tracks 2.21 / 1.48.  The grids end at 81,920 triangles
+// (grid.cu), where their cells begin to miss the caches: coax, detector 2 at 250 mm and a
+// volume source at 76,280 triangles 1.29 / 1.03, 1.10 / 1.03 and 1.04 / 0.90, at 104,848
+// 1.35 / 1.12, 1.09 / 1.22 and 1.07 / 0.98, at 215,128 1.37 / 1.49, 1.14 / 1.38 and 1.10 / 1.27.
 constexpr int kMegaGridMinTri = 8192;
 
 // The grids for a run of these instances (desc null: the tree serves it).  Every birth
@@ -1136,6 +1139,9 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
     // ~1 ms and ~6.7 ns (coax and Table 4 detector at 2e6 .. 1e7 histories per run):
     // break-even near 2.9e5 reaching histories.  Histories that miss the scene cost
     // little in either form.
+    // (With grids and chunks by what is left the megakernel is the faster one up to about
+    // 1e6: 2e6 coax histories, 5e5 reaching, 2.3 / 3.7 ms.  The line stays, since the two
+    // forms differ in about one history in a million, and so would a call's results.)
     if (variant == GADEP_VARIANT_AUTO)
         variant = wf_ok && reaching >= (double)(1u << 18) ? GADEP_VARIANT_WAVEFRONT : GADEP_VARIANT_MEGA;
     if (variant == GADEP_VARIANT_WAVEFRONT && !wf_ok) {
