@@ -31,6 +31,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -180,43 +181,48 @@ struct Words {
 // Per-block tallies in shared memory, one record per instance, flushed once per
 // launch into the block's tally copy: finished histories of many instances mix
 // in every launch, so per-thread accumulators would flush constantly.
+template <bool WIDE>
 struct STally {
-    unsigned int hist, fep, zero, over, err, seg, inter, errbits;
-    float dep, dep_all, esc;
-    unsigned int culled;
+    using Energy = std::conditional_t<WIDE, double, float>;
+    Energy dep, dep_all, esc;
+    unsigned int hist, fep, zero, over, err, seg, inter, errbits, culled;
 };
 
-template <bool GRAD>
+// GRAD: scores of the full-energy peak.  WIDE: the energies' sums in FP64, a warp's histories
+// at a time.  Where the trace kernel applies crossings more histories end in one launch of
+// physics, and FP32 block sums lose digits: sum_dep_active against the FP64 sum of the
+// histories' deposits, coax, rms of 12 runs, trace on trees with FP32 / on grids with FP32 /
+// on grids with FP64: 1e8 histories at 1332 keV 1.2e-9 / 2.2e-9 / 1.0e-10, 1e7 at 662 keV
+// 0.7e-9 / 1.5e-9 / 1.6e-10, with charged-particle tracks 1.1e-9 / 1.4e-9 / 0.4e-9 (physics of
+// 1e8 histories on grids 2.94 -> 3.10 ms).  Gradients, 6e6 histories: 1.7e-9 / 4.8e-9 / 2.1e-9
+// (physics 2.08 -> 1.99 ms; every lane adding in FP64 3.62).
+template <bool GRAD, bool WIDE>
 struct BlockTally {
-    STally *t;
-    double *sc;                 // GRAD: [n_inst][kSums] fep score sums and squares, then the energies' sums
-    static constexpr int kSums = 11;
+    using Tally = STally<WIDE>;
+    Tally *t;
+    double *sc;                 // GRAD: [n_inst][8] fep score sums and squares
     int n;
     __device__ void init(void *smem, int n_inst)
     {
-        t = reinterpret_cast<STally *>(smem);
+        t = reinterpret_cast<Tally *>(smem);
         sc = reinterpret_cast<double *>(t + n_inst);
         n = n_inst;
-        for (int i = threadIdx.x; i < n_inst; i += blockDim.x) t[i] = STally{ 0, 0, 0, 0, 0, 0, 0, 0, 0.f, 0.f, 0.f, 0u };
+        for (int i = threadIdx.x; i < n_inst; i += blockDim.x) t[i] = Tally{};
         if (GRAD)
-            for (int i = threadIdx.x; i < kSums * n_inst; i += blockDim.x) sc[i] = 0.0;
+            for (int i = threadIdx.x; i < 8 * n_inst; i += blockDim.x) sc[i] = 0.0;
     }
     // GRAD: the scores of a history in the full-energy peak
     __device__ void scores(int inst, const float *score)
     {
         for (int g = 0; g < 4; ++g) {
             const double v = (double)score[g];
-            atomicAdd(&sc[kSums * inst + g], v);
-            atomicAdd(&sc[kSums * inst + 4 + g], v * v);
+            atomicAdd(&sc[8 * inst + g], v);
+            atomicAdd(&sc[8 * inst + 4 + g], v * v);
         }
     }
     // The finished histories of a warp (every lane calls; fin: this lane finished
     // one): the lanes of one instance are summed in registers and one lane adds
     // the sums, instead of every lane adding its own.
-    // GRAD adds them in FP64: with crossings applied by the trace kernel more histories
-    // end in one launch, and FP32 block sums, a history at a time, put the deposits of
-    // runs of 6e6 histories 4.8e-9 off the FP64 value instead of 1.7e-9 (now 2.1e-9;
-    // physics of 1.2e7 histories 2.08 -> 1.99 ms, every lane adding in FP64 3.62).
     __device__ void history_warp(bool fin, int inst, uint32_t segs, uint32_t herr, bool fep, float edep,
                                  float dep_all, float esc, float e_max)
     {
@@ -244,23 +250,17 @@ struct BlockTally {
                 e += __shfl_xor_sync(FULL, e, o);
             }
             if (lane == src) {
-                STally &s = t[gi];
+                Tally &s = t[gi];
                 atomicAdd(&s.hist, (unsigned int)__popc(grp));
                 atomicAdd(&s.seg, seg);
                 if (n_err) { atomicAdd(&s.err, n_err); atomicOr(&s.errbits, eb); }
                 if (n_fep) atomicAdd(&s.fep, n_fep);
                 if (n_zero) atomicAdd(&s.zero, n_zero);
                 if (n_over) atomicAdd(&s.over, n_over);
-                if (GRAD) {
-                    double *sum = &sc[kSums * gi + 8];
-                    if (d != 0.0f) atomicAdd(&sum[0], (double)d);
-                    if (da != 0.0f) atomicAdd(&sum[1], (double)da);
-                    if (e != 0.0f) atomicAdd(&sum[2], (double)e);
-                } else {
-                    if (d != 0.0f) atomicAdd(&s.dep, d);
-                    if (da != 0.0f) atomicAdd(&s.dep_all, da);
-                    if (e != 0.0f) atomicAdd(&s.esc, e);
-                }
+                using Energy = typename Tally::Energy;
+                if (d != 0.0f) atomicAdd(&s.dep, (Energy)d);
+                if (da != 0.0f) atomicAdd(&s.dep_all, (Energy)da);
+                if (e != 0.0f) atomicAdd(&s.esc, (Energy)e);
             }
         }
     }
@@ -268,7 +268,7 @@ struct BlockTally {
     // deposited, the source energy escaped
     __device__ void culled(int inst, uint32_t n, float E0)
     {
-        STally &s = t[inst];
+        Tally &s = t[inst];
         atomicAdd(&s.hist, n);
         atomicAdd(&s.seg, n);
         atomicAdd(&s.zero, n);
@@ -279,7 +279,7 @@ struct BlockTally {
     {
         __syncthreads();
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const STally &s = t[i];
+            const Tally &s = t[i];
             if (!s.hist && !s.seg && !s.inter) continue;
             TallyDev &d = T[i];
             if (s.hist) atomicAdd(&d.n_hist, (unsigned long long)s.hist);
@@ -290,23 +290,22 @@ struct BlockTally {
             if (s.seg) atomicAdd(&d.n_segments, (unsigned long long)s.seg);
             if (s.inter) atomicAdd(&d.n_interactions, (unsigned long long)s.inter);
             if (s.culled) atomicAdd(&d.n_culled, (unsigned long long)s.culled);
-            const double *sum = GRAD ? &sc[kSums * i + 8] : nullptr;
-            atomicAdd(&d.sum_dep_active, GRAD ? sum[0] : (double)s.dep);
-            atomicAdd(&d.sum_dep_all, GRAD ? sum[1] : (double)s.dep_all);
-            atomicAdd(&d.sum_esc, GRAD ? sum[2] : (double)s.esc);
+            atomicAdd(&d.sum_dep_active, (double)s.dep);
+            atomicAdd(&d.sum_dep_all, (double)s.dep_all);
+            atomicAdd(&d.sum_esc, (double)s.esc);
             if (GRAD)
                 for (int g = 0; g < 4; ++g) {
-                    atomicAdd(&d.fep_score[g], sc[kSums * i + g]);
-                    atomicAdd(&d.fep_score_sq[g], sc[kSums * i + 4 + g]);
+                    atomicAdd(&d.fep_score[g], sc[8 * i + g]);
+                    atomicAdd(&d.fep_score_sq[g], sc[8 * i + 4 + g]);
                 }
         }
     }
 };
 
-template <bool GRAD>
+template <bool GRAD, bool WIDE>
 __host__ __device__ constexpr size_t block_tally_bytes(int n_inst)
 {
-    return (size_t)n_inst * (sizeof(STally) + (GRAD ? BlockTally<true>::kSums * sizeof(double) : 0));
+    return (size_t)n_inst * (sizeof(STally<WIDE>) + (GRAD ? 8 * sizeof(double) : 0));
 }
 
 struct Ctrl {
@@ -502,7 +501,7 @@ __global__ void __launch_bounds__(256) gen_kernel(const Params P, State S)
     extern __shared__ int4 smem_gen[];     // 16-byte aligned: the tallies hold FP64 sums
     __shared__ unsigned long long s_chunk, s_base;
     __shared__ unsigned int s_warp[8];
-    BlockTally<false> bt;               // culled histories carry no score
+    BlockTally<false, false> bt;               // culled histories carry no score
     bt.init(smem_gen, P.n_inst);
     const unsigned long long live0 = c.gen_live, tail0 = c.pend_tail;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1286,10 +1285,11 @@ __global__ void __launch_bounds__(128) left_kernel(const Params P, State S)
 // Bounds on registers: with room for three blocks of 256 per SM, ptxas allocates the
 // photon-only form without spilling in 64 registers (so four blocks still fit; under a
 // four-block bound it spilled a few bytes and ran slower) and the charged-particle form
-// in 80; the gradient form would take 69 and drop to three blocks per SM, slower than
-// its small spill at four, so it keeps the four-block bound.
+// in 80; the gradient form would take 69 and the photon form on grids (FP64 sums) 66, and
+// drop to three blocks per SM, slower than their small spills at four (36 and 8 bytes), so
+// they keep the four-block bound.
 template <bool GRAD, bool COUNT, bool EM, bool GRID>
-__global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params P, State S, int cur,
+__global__ void __launch_bounds__(256, GRAD || (GRID && !EM) ? 4 : 3) physics_kernel(const Params P, State S, int cur,
                                                       unsigned long long *counters)
 {
     const uint32_t FULL = 0xffffffffu;
@@ -1298,11 +1298,11 @@ __global__ void __launch_bounds__(256, GRAD ? 4 : 3) physics_kernel(const Params
     extern __shared__ int4 s_reg[];
     __shared__ unsigned int s_cnt[3], s_base[3];    // queue, free slots, deferred tracks
     for (int i = threadIdx.x; i < P.n_region; i += blockDim.x) s_reg[i] = P.regions[i];
-    BlockTally<GRAD> bt;
+    BlockTally<GRAD, GRAD || GRID> bt;
     bt.init(s_reg + P.n_region, P.n_inst);
     // key histogram of the next queue, after the block tallies
     unsigned int *s_hist = reinterpret_cast<unsigned int *>(
-        reinterpret_cast<char *>(s_reg + P.n_region) + block_tally_bytes<GRAD>(P.n_inst));
+        reinterpret_cast<char *>(s_reg + P.n_region) + block_tally_bytes<GRAD, GRAD || GRID>(P.n_inst));
     const int n_keys = P.n_keys;
     for (int k = threadIdx.x; k < n_keys; k += blockDim.x) s_hist[k] = 0u;
     if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
@@ -1772,12 +1772,15 @@ void wavefront_destroy(WavefrontBuffers *w)
     delete w;
 }
 
-// GRID matters to the charged-particle form alone: the others trace nothing.
+// GRID: the energies' sums in FP64, and the charged-particle form's tracks on grids; the
+// gradient form is the same with and without.
 static const void *physics_of(bool grad, bool count, bool em, bool grid)
 {
     using namespace wf;
     if (grad) return count ? (const void *)physics_kernel<true, true, false, false>
                            : (const void *)physics_kernel<true, false, false, false>;
+    if (!em && grid) return count ? (const void *)physics_kernel<false, true, false, true>
+                                  : (const void *)physics_kernel<false, false, false, true>;
     if (!em) return count ? (const void *)physics_kernel<false, true, false, false>
                           : (const void *)physics_kernel<false, false, false, false>;
     if (grid) return count ? (const void *)physics_kernel<false, true, true, true>
@@ -1814,11 +1817,13 @@ gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P0, bool grad
         return fail(GADEP_E_INVAL, "wavefront: at most %d instances per run", kWavefrontMaxInstances);
     if (!wavefront_supports(P.n_region, 0)) return fail(GADEP_E_INVAL, "wavefront: too many regions");
     // dynamic shared memory: block tallies (gen); region table + block tallies (physics)
-    const size_t gsm = wf::block_tally_bytes<false>(P.n_inst);
+    const size_t gsm = wf::block_tally_bytes<false, false>(P.n_inst);
     const size_t ksm = (size_t)P.n_keys * sizeof(unsigned int);   // key histogram (spawn)
     const size_t ssm = 2 * ksm;                                    // bucket starts and counts (sort)
     const size_t rsm = (size_t)P.n_region * sizeof(int4) +
-                       (grad ? wf::block_tally_bytes<true>(P.n_inst) : wf::block_tally_bytes<false>(P.n_inst)) +
+                       (grad ? wf::block_tally_bytes<true, true>(P.n_inst)
+                             : P.grid.desc ? wf::block_tally_bytes<false, true>(P.n_inst)
+                                           : wf::block_tally_bytes<false, false>(P.n_inst)) +
                        (size_t)P.n_keys * sizeof(unsigned int);
     {
         cudaError_t e = cudaSuccess;
