@@ -250,9 +250,9 @@ __device__ __forceinline__ float back_from_reciprocal(float d)
 // Nearest triangle of grid g along o + t d with t_min < t < t_max (exclusive), skipping
 // mesh triangle `exclude`: its mesh triangle id or -1; t_hit and entering set on a hit.
 // The selection and the distance are those of traverse() in device_common.cuh, but where
-// two triangles tie for the nearest hit, whose order of tests decides.  t_min >= 0.
-// LEAVE: such queries are left to the tree (`left` set, no hit).
-template <bool COUNT, bool LEAVE>
+// two triangles tie for the nearest hit, whose order of tests decides: such queries are
+// left to the tree (`left` set, no hit).  t_min >= 0.
+template <bool COUNT>
 __device__ __forceinline__ int grid_query(const GridSet &G, const float4 *__restrict__ planes, int g, float ox, float oy,
                                           float oz, float dx, float dy, float dz, float t_min, int exclude,
                                           float &t_hit, bool &entering, bool &left, TravStats &st,
@@ -289,14 +289,14 @@ __device__ __forceinline__ int grid_query(const GridSet &G, const float4 *__rest
     }
     if (COUNT) { st.nodes += nn; st.boxes += nn; st.tris += nt; }
     if (h.best < 0) return -1;
-    if (LEAVE && (h.best & kTied) != 0) {
+    if ((h.best & kTied) != 0) {
         left = true;
         return -1;
     }
     t_hit = nearest_t(planes, h, ox, oy, oz, back_from_reciprocal(dx), back_from_reciprocal(dy),
                       back_from_reciprocal(dz), t_min);
     entering = (h.best & 1) != 0;
-    return (h.best & (kTied - 1)) >> 1;
+    return h.best >> 1;
 }
 
 }  // namespace dev

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                 bool reloc = false, by_tree = !GRID;
                 while (true) {
                     if (!by_tree) {
-                        hit = grid_query<COUNT, true>(P.grid, P.planes, reloc ? P.grid.all : region, ox, oy, oz, dx, dy, dz,
+                        hit = grid_query<COUNT>(P.grid, P.planes, reloc ? P.grid.all : region, ox, oy, oz, dx, dy, dz,
                                                 t_cur, last_tri, t_hit, entering, by_tree, ts);
                         if (by_tree) continue;          // left to the tree
                     } else {
