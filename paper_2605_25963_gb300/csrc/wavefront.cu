@@ -1078,7 +1078,7 @@ __global__ void __launch_bounds__(256, 4) trace_grid_kernel(const Params P, Stat
             continue;
         }
         if (!m_done && !n_idle) break;           // nothing is left: serve is set by m_test | m_step == 0
-        bool begin = false;
+        bool begin = false, leave = false;
         // ---- queries that are done: cross, relocate, or store the hit ----
         if (has && word == 0) {
             const int where = L.where[lane], region = where & 255;
@@ -1131,7 +1131,7 @@ __global__ void __launch_bounds__(256, 4) trace_grid_kernel(const Params P, Stat
                 ht.region = treg;
                 ht.code = kCodeBias + (best >= 0 ? (ent ? 1 : 0) + (reloc ? kRelocated : 0)
                                                  : (reloc ? kRelocated : (bounded ? kBeyond : 0)));
-                if (left_out) S.left[atomicAdd(&S.ctrl->n_left, 1u)] = qidx;
+                leave = left_out;
                 ht.code |= crossed << kCodeBits;
                 S.hit[qidx] = ht;
                 if (crossed)
@@ -1139,6 +1139,13 @@ __global__ void __launch_bounds__(256, 4) trace_grid_kernel(const Params P, Stat
                 has = false;
                 reloc = false;
             }
+        }
+        const uint32_t m_leave = __ballot_sync(FULL, leave);
+        if (m_leave) {
+            unsigned int at = 0;
+            if (lane == 0) at = atomicAdd(&S.ctrl->n_left, (unsigned int)__popc(m_leave));
+            at = __shfl_sync(FULL, at, 0) + __popc(m_leave & ((1u << lane) - 1u));
+            if (leave) S.left[at] = L.qidx[lane];
         }
         // ---- dynamic fetch: lanes without a ray take the next queue entries ----
         const uint32_t need = __ballot_sync(FULL, !has);
@@ -1240,8 +1247,11 @@ static __device__ __noinline__ TreeHit tree_nearest(const float4 *nodes, const f
                     (err & ERR_STACK) ? -2 : (entering ? 1 : 0) };
 }
 
-// The queries that trace_grid_kernel left to the tree (two triangles at one distance:
-// about one query in 10^7), one per thread, at the segment where it left them.
+// The queries that trace_grid_kernel left to the tree (two triangles at one distance: about
+// one query in 10^7, but every crossing of two surfaces that coincide), one per thread, at
+// the segment where it left them.  As many blocks as SMs hold at once: a pencil of 1e6
+// photons along an edge of the coax took 513 ms with one block, 11.7 with these, 14.0 with a
+// quarter of them; runs without ties the same with any.
 __global__ void __launch_bounds__(128) left_kernel(const Params P, State S)
 {
     const unsigned int n = S.ctrl->n_left;
@@ -1886,7 +1896,7 @@ gadep_status wavefront_run(WavefrontBuffers *w, const dev::Params &P0, bool grad
             grid = dim3(w->trace_grid);
             smem = P.grid.desc ? (size_t)P.n_region * sizeof(int4) : 0;
             args[0] = &P; args[1] = &S; args[2] = &c; args[3] = &counters; break;
-        case KK_N + 5: fn = (const void *)wf::left_kernel; block = dim3(128);
+        case KK_N + 5: fn = (const void *)wf::left_kernel; grid = dim3(w->work_grid / 2); block = dim3(128);
             args[0] = &P; args[1] = &S; break;
         case KK_PHYSICS:
             fn = physics_of(grad, count, P.e_model != 0, P.grid.desc != nullptr);
