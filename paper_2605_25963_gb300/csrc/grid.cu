@@ -1,11 +1,10 @@
 // grid.cu -- builds the uniform grids of grid.cuh on the device, once per mesh.
 //
-// One warp per (triangle, grid) pair walks the cells of the triangle's box and keeps
-// those that the triangle meets (separating axes, FP64, cells grown by kGridPad):
-// a first pass counts, a prefix sum over the cells places the lists, a second pass
-// fills them, and each list is put in the order of the triangle ids.  The distances
-// to the nearest occupied cell follow axis by axis (the Chebyshev distance is
-// separable).
+// A warp walks the cells of a triangle's box in a grid and keeps those that the triangle
+// meets (separating axes, cells grown by kGridPad): a first pass counts, a prefix sum over
+// the cells places the lists, a second pass fills them, and each list is put in the order
+// of the triangle ids.  The distances to the nearest occupied cell follow axis by axis (the
+// Chebyshev distance is separable).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -27,81 +26,100 @@ constexpr double kMinCells = 131072.0, kMaxCells = 4194304.0;  // per grid; indi
 constexpr unsigned long long kMaxTotal = 1ull << 27;           // cells of all grids (2.4 GB while they are built)
 constexpr int kMinTris = 2048, kMaxTris = 5 << 14;      // no run walks the grids of other meshes
 constexpr int kMaxSkip = 64;
+constexpr int kWarpCells = 4096;            // of a triangle's box, by one warp; larger boxes take more warps
+// Cells of the triangles' boxes, on average over the triangles of all grids, at most.  Detectors
+// have 200 to 600, lying obliquely 1,400; a tilted cylinder of 600 long triangles a side has
+// 20,000 (2 x 0.6 ms, its trees 11).  Large triangles that lie obliquely have up to the 4e6 of
+// a grid: 80,000 of them would take 4 s a pass (the trees 0.35), at this limit 60 ms.
+constexpr double kMaxBox = 65536.0;
 
 struct GridDesc {                           // host and build kernels
-    double lo[3], s[3];
+    double lo[3], s[3], inv[3];             // inv: 1 / s
     int n[3];
     uint32_t off;                           // first cell
 };
 
-struct Pair { int32_t tri, grid; };
+// A triangle in a grid; the part of its box that a warp walks.
+struct Pair { int32_t tri; uint16_t grid, part; };
 
-__device__ bool separated(const double v[3][3], double ax, double ay, double az, const double h[3])
+// Whether the projections of triangle v on the axis (x, y) miss those of the box of half
+// extent h round the origin.
+__device__ __forceinline__ bool separated(const float v[3][3], int a, int b, float x, float y, float h)
 {
-    const double p0 = v[0][0] * ax + v[0][1] * ay + v[0][2] * az, p1 = v[1][0] * ax + v[1][1] * ay + v[1][2] * az,
-                 p2 = v[2][0] * ax + v[2][1] * ay + v[2][2] * az;
-    const double r = h[0] * fabs(ax) + h[1] * fabs(ay) + h[2] * fabs(az);
-    return fmin(p0, fmin(p1, p2)) > r || fmax(p0, fmax(p1, p2)) < -r;
-}
-
-// Triangle v (relative to the box centre) against the box of half extents h; the
-// axes along the coordinates are settled by the caller's cell range.
-__device__ bool meets(const double v[3][3], const double h[3])
-{
-    double e[3][3];
-    for (int k = 0; k < 3; ++k)
-        for (int a = 0; a < 3; ++a) e[k][a] = v[(k + 1) % 3][a] - v[k][a];
-    if (separated(v, e[0][1] * e[1][2] - e[0][2] * e[1][1], e[0][2] * e[1][0] - e[0][0] * e[1][2],
-                  e[0][0] * e[1][1] - e[0][1] * e[1][0], h))
-        return false;
-    for (int k = 0; k < 3; ++k)
-        if (separated(v, 0.0, -e[k][2], e[k][1], h) || separated(v, e[k][2], 0.0, -e[k][0], h) ||
-            separated(v, -e[k][1], e[k][0], 0.0, h))
-            return false;
-    return true;
+    const float p0 = fmaf(v[0][a], x, v[0][b] * y), p1 = fmaf(v[1][a], x, v[1][b] * y), p2 = fmaf(v[2][a], x, v[2][b] * y);
+    const float r = h * (fabsf(x) + fabsf(y));
+    return fminf(p0, fminf(p1, p2)) > r || fmaxf(p0, fmaxf(p1, p2)) < -r;
 }
 
 // Entries of a list of c ids: rounded up to fours, one more for the length of a long one.
 constexpr uint32_t kLong = 127;
 __host__ __device__ inline uint32_t padded(uint32_t c) { return (c + (c >= kLong ? 4u : 3u)) & ~3u; }
 
-// FILL 0: counts[cell] += 1 per triangle that meets it; 1: the ids go to
+// list null: counts[cell] += 1 per triangle that meets it; otherwise the ids go to
 // list[start[cell] + counts[cell]++] (behind the length where the cell has kLong or more).
-template <int FILL>
+// One kernel for both, so that both find the same cells to the last bit.
+// In FP32 and cells, with the triangle's lowest cell as the origin: coordinates of at most 160
+// are then good to 2e-5 of a cell, and kSlack more than covers the tests' rounding (the
+// normal's, which a sliver's cancels, is added by itself): 0.2 % more cells than in FP64, none
+// fewer.  Bound by issue, 2.5e11 cells of boxes a second.  FP64 throughout, a triangle to a
+// warp, took 2.8 ms a pass on 3,456 triangles, most of it one warp with the largest box, and
+// 3.1 on 20,088: now 0.14 and 0.29 (counting), 0.22 and 0.36 (lists).
+constexpr float kSlack = 1e-3f;
 __global__ void __launch_bounds__(256) raster_kernel(const Pair *pairs, long long n_pairs, const GridDesc *grids,
                                                      const float4 *tris, uint32_t *counts, const uint32_t *totals,
                                                      const uint32_t *start, uint32_t *list)
 {
     const int lane = threadIdx.x & 31;
     const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
+    constexpr float h = 0.5f + (float)kGridPad + kSlack;
     for (long long p = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < n_pairs; p += n_warps) {
-        const int tri = pairs[p].tri;
-        const GridDesc &g = grids[pairs[p].grid];
-        double v[3][3], h[3];
+        const Pair pair = pairs[p];
+        const GridDesc &g = grids[pair.grid];
+        float v[3][3], far = 0.0f;
         int a0[3], na[3];
-        for (int k = 0; k < 3; ++k) {
-            const float4 q = tris[3 * (size_t)tri + k];
-            v[k][0] = q.x; v[k][1] = q.y; v[k][2] = q.z;
+        const float4 q0 = tris[3 * (size_t)pair.tri], q1 = tris[3 * (size_t)pair.tri + 1], q2 = tris[3 * (size_t)pair.tri + 2];
+        for (int a = 0; a < 3; ++a) {
+            const double inv = g.inv[a];
+            const double x0 = ((double)(a == 0 ? q0.x : (a == 1 ? q0.y : q0.z)) - g.lo[a]) * inv,
+                         x1 = ((double)(a == 0 ? q1.x : (a == 1 ? q1.y : q1.z)) - g.lo[a]) * inv,
+                         x2 = ((double)(a == 0 ? q2.x : (a == 1 ? q2.y : q2.z)) - g.lo[a]) * inv;
+            a0[a] = max(1, (int)floor(fmin(x0, fmin(x1, x2)) - kGridPad));
+            na[a] = min(g.n[a] - 2, (int)floor(fmax(x0, fmax(x1, x2)) + kGridPad)) - a0[a] + 1;
+            v[0][a] = (float)(x0 - a0[a]);
+            v[1][a] = (float)(x1 - a0[a]);
+            v[2][a] = (float)(x2 - a0[a]);
+            far = fmaxf(far, (float)na[a] + 1.0f);
+        }
+        float e[3][3], n[3], e2[2] = { 0.0f, 0.0f }, rn = 0.0f;
+        for (int a = 0; a < 3; ++a) {
+            e[0][a] = v[1][a] - v[0][a];
+            e[1][a] = v[2][a] - v[1][a];
+            e[2][a] = v[0][a] - v[2][a];
+            e2[0] = fmaf(e[0][a], e[0][a], e2[0]);
+            e2[1] = fmaf(e[1][a], e[1][a], e2[1]);
         }
         for (int a = 0; a < 3; ++a) {
-            const double pad = kGridPad * g.s[a];
-            const double lo = fmin(v[0][a], fmin(v[1][a], v[2][a])) - pad, hi = fmax(v[0][a], fmax(v[1][a], v[2][a])) + pad;
-            a0[a] = max(1, (int)floor((lo - g.lo[a]) / g.s[a]));
-            na[a] = min(g.n[a] - 2, (int)floor((hi - g.lo[a]) / g.s[a])) - a0[a] + 1;
-            h[a] = 0.5 * g.s[a] + pad;
+            n[a] = e[0][(a + 1) % 3] * e[1][(a + 2) % 3] - e[0][(a + 2) % 3] * e[1][(a + 1) % 3];
+            rn = fmaf(h, fabsf(n[a]), rn);
         }
-        const long long cells = (long long)na[0] * na[1] * na[2];
-        for (long long i = lane; i < cells; i += 32) {
-            const int x = a0[0] + (int)(i % na[0]), y = a0[1] + (int)(i / na[0] % na[1]),
-                      z = a0[2] + (int)(i / ((long long)na[0] * na[1]));
-            const double c[3] = { g.lo[0] + (x + 0.5) * g.s[0], g.lo[1] + (y + 0.5) * g.s[1], g.lo[2] + (z + 0.5) * g.s[2] };
-            double w[3][3];
+        rn = fmaf(1e-6f * far, sqrtf(e2[0] * e2[1]), rn);
+        const long long cells = (long long)na[0] * na[1] * na[2], first = (long long)pair.part * kWarpCells,
+                        end = min(cells, first + kWarpCells);
+        for (int i = (int)first + lane; i < (int)end; i += 32) {
+            const int x = i % na[0], y = i / na[0] % na[1], z = i / (na[0] * na[1]);
+            const float c[3] = { (float)x + 0.5f, (float)y + 0.5f, (float)z + 0.5f };
+            float w[3][3];
             for (int k = 0; k < 3; ++k)
                 for (int a = 0; a < 3; ++a) w[k][a] = v[k][a] - c[a];
-            if (!meets(w, h)) continue;
-            const size_t cell = (size_t)g.off + ((size_t)z * g.n[1] + y) * g.n[0] + x;
+            if (fabsf(fmaf(n[0], w[0][0], fmaf(n[1], w[0][1], n[2] * w[0][2]))) > rn) continue;
+            bool apart = false;
+            for (int k = 0; k < 3; ++k)
+                apart = apart || separated(w, 1, 2, -e[k][2], e[k][1], h) || separated(w, 0, 2, e[k][2], -e[k][0], h) ||
+                        separated(w, 0, 1, -e[k][1], e[k][0], h);
+            if (apart) continue;
+            const size_t cell = (size_t)g.off + ((size_t)(a0[2] + z) * g.n[1] + (a0[1] + y)) * g.n[0] + (a0[0] + x);
             const uint32_t at = atomicAdd(&counts[cell], 1u);
-            if (FILL) list[start[cell] + (totals[cell] >= kLong ? 1u : 0u) + at] = (uint32_t)tri;
+            if (list) list[start[cell] + (totals[cell] >= kLong ? 1u : 0u) + at] = (uint32_t)pair.tri;
         }
     }
 }
@@ -234,7 +252,7 @@ void grid_free(gadep_bvh *b)
 
 // Builds the grids of b (device current).  Where they do not suit the mesh (coordinates
 // too coarse for the cells' margin, lists too long for the cell words, too few or too many
-// triangles) or leave no memory, the tree serves alone; b->d_grid stays null.
+// triangles, or mostly as large as the grids) or leave no memory, the tree serves alone; b->d_grid stays null.
 gadep_status grid_build(gadep_bvh *b)
 {
     const MeshData &m = b->geo;
@@ -246,6 +264,7 @@ gadep_status grid_build(gadep_bvh *b)
     sets.push_back(all);
     const size_t ng = sets.size();
     std::vector<float> rec(12 * (size_t)nt);
+    std::vector<float> low(3 * (size_t)nt, INFINITY), high(3 * (size_t)nt, -INFINITY);   // the triangles' boxes
     double far = 0.0;
     for (int t = 0; t < nt; ++t)
         for (int k = 0; k < 3; ++k) {
@@ -253,6 +272,8 @@ gadep_status grid_build(gadep_bvh *b)
                 const float x = (float)m.xyz[3 * (size_t)m.tri[3 * (size_t)t + k] + a];
                 rec[12 * (size_t)t + 4 * k + a] = x;
                 far = std::max(far, (double)std::fabs(x));
+                low[3 * (size_t)t + a] = std::min(low[3 * (size_t)t + a], x);
+                high[3 * (size_t)t + a] = std::max(high[3 * (size_t)t + a], x);
             }
             const int32_t w = k == 0 ? m.tri_solid[(size_t)t] + 1 : 0;
             std::memcpy(&rec[12 * (size_t)t + 4 * k + 3], &w, 4);
@@ -260,22 +281,19 @@ gadep_status grid_build(gadep_bvh *b)
     std::vector<GridDesc> desc(ng);
     std::vector<Pair> pairs;
     unsigned long long total = 0;
-    double pad = INFINITY;
+    double pad = INFINITY, left = 0.0;       // cells of boxes that may still come
+    for (const auto &set : sets) left += kMaxBox * (double)set.size();
     for (size_t r = 0; r < ng; ++r) {
         GridDesc &g = desc[r];
         std::memset(&g, 0, sizeof(g));
         g.off = (uint32_t)total;
         if (sets[r].empty()) continue;
         double lo[3] = { INFINITY, INFINITY, INFINITY }, hi[3] = { -INFINITY, -INFINITY, -INFINITY };
-        for (int32_t t : sets[r]) {
-            pairs.push_back(Pair{ t, (int32_t)r });
-            for (int k = 0; k < 3; ++k)
-                for (int a = 0; a < 3; ++a) {
-                    const double x = rec[12 * (size_t)t + 4 * k + a];
-                    lo[a] = std::min(lo[a], x);
-                    hi[a] = std::max(hi[a], x);
-                }
-        }
+        for (int32_t t : sets[r])
+            for (int a = 0; a < 3; ++a) {
+                lo[a] = std::min(lo[a], (double)low[3 * (size_t)t + a]);
+                hi[a] = std::max(hi[a], (double)high[3 * (size_t)t + a]);
+            }
         double vol = 1.0, longest = 0.0;
         for (int a = 0; a < 3; ++a) longest = std::max(longest, hi[a] - lo[a]);
         for (int a = 0; a < 3; ++a) vol *= std::max(hi[a] - lo[a], 1e-3 * longest);
@@ -286,12 +304,22 @@ gadep_status grid_build(gadep_bvh *b)
                 const double n = std::floor((hi[a] - lo[a]) / s + 0.1) + 3.0;   // a border cell on each side
                 g.n[a] = (int)std::min(n, 1e6);
                 g.s[a] = s;
+                g.inv[a] = 1.0 / s;
                 g.lo[a] = 0.5 * (lo[a] + hi[a]) - 0.5 * g.n[a] * s;
                 cells *= n;
             }
             if (cells <= kMaxCells) break;
         }
         pad = std::min(pad, kGridPad * g.s[0]);
+        // a box has at most two cells more along each axis than its length goes into whole ones
+        for (int32_t t : sets[r]) {
+            double box = 1.0;
+            for (int a = 0; a < 3; ++a)
+                box *= std::min((high[3 * (size_t)t + a] - low[3 * (size_t)t + a]) * g.inv[a] + 3.0, (double)g.n[a]);
+            if ((left -= box) < 0.0) return GADEP_OK;
+            for (int part = 0; part * (double)kWarpCells < box; ++part)
+                pairs.push_back(Pair{ t, (uint16_t)r, (uint16_t)part });
+        }
         total += (unsigned long long)g.n[0] * g.n[1] * g.n[2];
     }
     // the rounding of a position |x| away from the coordinate origin is a few units of
@@ -330,7 +358,7 @@ gadep_status grid_build(gadep_bvh *b)
     unsigned long long entries = 0;
     bool fits = true;
     if (e == cudaSuccess) {
-        raster_kernel<0><<<blocks, 256>>>(d_pairs, (long long)pairs.size(), d_desc, tris, counts, nullptr, nullptr, nullptr);
+        raster_kernel<<<blocks, 256>>>(d_pairs, (long long)pairs.size(), d_desc, tris, counts, nullptr, nullptr, nullptr);
         scan_kernel<<<tiles, kScanBlock>>>(counts, start, total, sums);
         e = cudaMemcpy(tile.data(), sums, tiles * 4, cudaMemcpyDeviceToHost);
         for (uint32_t &t : tile) {
@@ -368,7 +396,7 @@ gadep_status grid_build(gadep_bvh *b)
         if (e == cudaSuccess) e = alloc(&list, (size_t)entries);
         if (e == cudaSuccess) {
             const dim3 by_grid(512, (unsigned)ng);
-            raster_kernel<1><<<blocks, 256>>>(d_pairs, (long long)pairs.size(), d_desc, tris, cursor, counts, start, list);
+            raster_kernel<<<blocks, 256>>>(d_pairs, (long long)pairs.size(), d_desc, tris, cursor, counts, start, list);
             lists_kernel<<<by_grid, 256>>>(d_desc, counts, start, list, cells);
             distance_kernel<0><<<by_grid, 256>>>(d_desc, counts, nullptr, dist, nullptr);
             distance_kernel<1><<<by_grid, 256>>>(d_desc, counts, dist, dist + total, nullptr);

@@ -1,0 +1,80 @@
+"""Building the grids of meshes whose triangles are long or large and lie obliquely: their
+boxes hold most of a grid's cells.  A build with a device copy may take twice the time of
+the host's part (the trees) and 5 ms, the best of three each."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2605_25963_gb300 import api
+from paper_2605_25963_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from test_gpu_grid_ties import MEGA, box, on_grids_and_on_trees  # noqa: E402
+
+A, B = np.cos(0.7), np.sin(0.7)
+C, D = np.cos(0.9), np.sin(0.9)
+TILT = np.array([[A, -B, 0], [B, A, 0], [0, 0, 1]]) @ np.array([[1, 0, 0], [0, C, -D], [0, D, C]])
+
+
+def revolved(n, profile):
+    """The solid that a profile of (radius, z) from the lower to the upper end encloses."""
+    ang = 2.0 * np.pi * np.arange(n) / n
+    xyz = [(0.0, 0.0, profile[0][1])] + [(r * np.cos(a), r * np.sin(a), z) for r, z in profile for a in ang] + \
+          [(0.0, 0.0, profile[-1][1])]
+    at = lambda j, i: 1 + j * n + i % n
+    tri = []
+    for i in range(n):
+        tri += [(0, at(0, i + 1), at(0, i)), (len(xyz) - 1, at(len(profile) - 1, i), at(len(profile) - 1, i + 1))]
+        for j in range(len(profile) - 1):
+            tri += [(at(j, i), at(j, i + 1), at(j + 1, i + 1)), (at(j, i), at(j + 1, i + 1), at(j + 1, i))]
+    return np.array(xyz), np.array(tri, np.int32)
+
+
+def solids(parts, active):
+    xyz, tri, solid, base = [], [], [], 0
+    for s, (x, t) in enumerate(parts):
+        xyz.append(x @ TILT.T)
+        tri.append(t + base)
+        solid.append(np.full(len(t), s, np.int32))
+        base += len(x)
+    n = len(parts)
+    return api.detmesh_from_arrays(np.concatenate(xyz).astype(np.float32), np.concatenate(tri), np.concatenate(solid),
+                                   [W.MAT_GE] * n, active, [-1] * n)
+
+
+def best(f):
+    out = []
+    for _ in range(3):
+        t = time.perf_counter()
+        f()
+        out.append(time.perf_counter() - t)
+    return min(out)
+
+
+@pytest.mark.parametrize("name", ["long", "large"])
+def test_oblique_triangles_do_not_hold_up_the_build(name):
+    if name == "long":
+        mesh = solids([revolved(600, [(30.0, 0.0), (30.0, 60.0)])], [1])
+    else:       # 200 boxes, each within the one before
+        half = [30.0 - 0.1 * k for k in range(200)]
+        mesh = solids([box((-h, -h, -h), (h, h, h), 1) for h in half], [1] * 200)
+    api.gadep_bvh_build(mesh, 0)
+    host, device = best(lambda: api.gadep_bvh_build(mesh, -1)), best(lambda: api.gadep_bvh_build(mesh, 0))
+    assert device <= 2.0 * host + 5e-3, (host, device)
+
+
+def test_oblique_mesh_on_grids_matches_the_trees():
+    rings = [(7.0, 0.0), (14.0, 0.0), (22.0, 0.0)] + [(30.0, 60.0 * k / 8) for k in range(9)] + [(22.0, 60.0), (14.0, 60.0), (7.0, 60.0)]
+    inner = [(0.9 * r, 1.0 + 0.95 * z) for r, z in rings]
+    bvh = api.gadep_bvh_build(solids([revolved(150, rings), revolved(150, inner)], [0, 1]), 0)
+    assert bvh.stats()["n_tri"] >= 8192
+    src = W.Source(kind=W.SRC_POINT, pos=tuple(float(v) for v in TILT @ np.array([3.0, 2.0, 90.0])))
+    grids, trees = on_grids_and_on_trees(bvh, src, 662.0, 500_000, variant=MEGA)
+    assert grids[0] < 1.5 < trees[0]
+    assert grids[1] == trees[1] and grids[1][4] == 0
+    assert np.array_equal(grids[2], trees[2])
