@@ -152,16 +152,20 @@ __global__ void __launch_bounds__(kScanBlock) scan_kernel(const uint32_t *in, ui
 }
 
 // Puts each list in the order of the ids (heap sort: a fan's centre may hold thousands)
-// and writes the words of the occupied cells (one grid per blockIdx.y).
+// and writes the words of the occupied cells (one grid per blockIdx.y).  sums: of the lists'
+// lengths and of their squares, per grid.
 __global__ void __launch_bounds__(256) lists_kernel(const GridDesc *grids, const uint32_t *counts, const uint32_t *start,
-                                                    uint32_t *list, int *cells)
+                                                    uint32_t *list, int *cells, unsigned long long *sums)
 {
+    unsigned long long length = 0, square = 0;
     const GridDesc &g = grids[blockIdx.y];
     const uint32_t n = (uint32_t)g.n[0] * g.n[1] * g.n[2], first = n ? start[g.off] : 0u;
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const size_t i = (size_t)g.off + k;
         const uint32_t c = counts[i];
         if (!c) continue;
+        length += c;
+        square += (unsigned long long)c * c;
         uint32_t *l = list + start[i];
         if (c >= kLong) *l++ = c;
         for (uint32_t end = c, root = c / 2; end > 1u;) {
@@ -183,6 +187,14 @@ __global__ void __launch_bounds__(256) lists_kernel(const GridDesc *grids, const
             l[at] = x;
         }
         cells[i] = (int)(0x80000000u | min(c, kLong) << 24 | (start[i] - first) / 4u);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        length += __shfl_xor_sync(0xffffffffu, length, o);
+        square += __shfl_xor_sync(0xffffffffu, square, o);
+    }
+    if ((threadIdx.x & 31) == 0 && length) {
+        atomicAdd(&sums[2 * blockIdx.y], length);
+        atomicAdd(&sums[2 * blockIdx.y + 1], square);
     }
 }
 
@@ -247,7 +259,7 @@ void grid_free(gadep_bvh *b)
     cudaFree(b->d_grid);
     cudaFree(b->d_grid_list);
     b->d_grid = b->d_grid_list = nullptr;
-    b->grid_safe = 0.0f;
+    b->grid_safe = b->grid_crowd = 0.0f;
 }
 
 // Builds the grids of b (device current).  Where they do not suit the mesh (coordinates
@@ -335,6 +347,7 @@ gadep_status grid_build(gadep_bvh *b)
     Pair *d_pairs = nullptr;
     uint32_t *counts = nullptr, *cursor = nullptr, *start = nullptr, *sums = nullptr, *list = nullptr;
     uint8_t *dist = nullptr;
+    unsigned long long *lengths = nullptr;
     float4 *tris = nullptr;
     const uint32_t tiles = (uint32_t)((total + kScanTile - 1) / kScanTile);
     cudaError_t e = alloc(&base, o_tris + (size_t)nt * 9 * sizeof(float4));
@@ -346,15 +359,18 @@ gadep_status grid_build(gadep_bvh *b)
     if (e == cudaSuccess) e = alloc(&sums, tiles);
     if (e == cudaSuccess) e = alloc(&dist, 2 * total);
     if (e == cudaSuccess) e = alloc(&tris, (size_t)nt * 3);
+    if (e == cudaSuccess) e = alloc(&lengths, 2 * ng);
     if (e == cudaSuccess) e = cudaMemcpy(d_desc, desc.data(), ng * sizeof(GridDesc), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(d_pairs, pairs.data(), pairs.size() * sizeof(Pair), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(tris, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(counts, 0, total * 4);
     if (e == cudaSuccess) e = cudaMemset(cursor, 0, total * 4);
+    if (e == cudaSuccess) e = cudaMemset(lengths, 0, 2 * ng * sizeof(*lengths));
     int *cells = (int *)(base + o_cells);
     const int blocks = (int)std::min<size_t>(65535, (pairs.size() + 7) / 8);
     const unsigned cell_blocks = (unsigned)((total + 255) / 256);
     std::vector<uint32_t> tile(tiles), first(ng + 1);
+    std::vector<unsigned long long> sum(2 * ng, 0);
     unsigned long long entries = 0;
     bool fits = true;
     if (e == cudaSuccess) {
@@ -397,13 +413,14 @@ gadep_status grid_build(gadep_bvh *b)
         if (e == cudaSuccess) {
             const dim3 by_grid(512, (unsigned)ng);
             raster_kernel<<<blocks, 256>>>(d_pairs, (long long)pairs.size(), d_desc, tris, cursor, counts, start, list);
-            lists_kernel<<<by_grid, 256>>>(d_desc, counts, start, list, cells);
+            lists_kernel<<<by_grid, 256>>>(d_desc, counts, start, list, cells, lengths);
             distance_kernel<0><<<by_grid, 256>>>(d_desc, counts, nullptr, dist, nullptr);
             distance_kernel<1><<<by_grid, 256>>>(d_desc, counts, dist, dist + total, nullptr);
             distance_kernel<2><<<by_grid, 256>>>(d_desc, counts, dist + total, nullptr, cells);
             permute_kernel<<<(3 * nt + 255) / 256, 256>>>(tris, nt, (float4 *)(base + o_tris));
             e = cudaGetLastError();
         }
+        if (e == cudaSuccess) e = cudaMemcpy(sum.data(), lengths, sum.size() * sizeof(sum[0]), cudaMemcpyDeviceToHost);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
     }
     cudaFree(d_desc);
@@ -414,6 +431,7 @@ gadep_status grid_build(gadep_bvh *b)
     cudaFree(sums);
     cudaFree(dist);
     cudaFree(tris);
+    cudaFree(lengths);
     if (e != cudaSuccess || !list) {
         cudaFree(base);
         cudaFree(list);
@@ -427,6 +445,9 @@ gadep_status grid_build(gadep_bvh *b)
     b->grid_cells = o_cells;
     b->grid_tris = o_tris;
     b->grid_safe = (float)safe;
+    b->grid_crowd = 0.0f;
+    for (size_t r = 0; r + 1 < ng; ++r)             // the grid of every triangle serves few queries
+        if (sum[2 * r]) b->grid_crowd = std::max(b->grid_crowd, (float)((double)sum[2 * r + 1] / (double)sum[2 * r]));
     return GADEP_OK;
 }
 

@@ -1211,10 +1211,17 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
         // the tree is a few nodes (192 triangles 2.80 / 3.37), on large ones the cells miss
         // the caches (25,112 triangles, 1.5e6 reaching 5.38 / 5.52; 76,280 triangles, 7.5e6
         // reaching 14.5 / 15.8); a plain volume source gains 2 % at best.
+        // Where triangles crowd in a few cells (end faces that are fans: 10 and more to a
+        // list that an entry is in, on average; rings have 3 to 9) one lane's long list
+        // holds up each iteration.  Such meshes need 2^23 that reach: nested cans with fans of
+        // 256, 1.1e6 reaching 6.19 / 7.50, 3e6 10.0 / 10.8, 1e7 23.9 / 18.2; one can with fans
+        // of 1,200, 1.8e6 reaching 9.4 / 14.4, 6e6 21.1 / 20.3; with tracks 1.8e5 6.7 / 9.5.
         const int n_tri = b->geo.n_tri();
-        const bool walks = electrons ? n_tri >= 2048 && n_tri <= 49152
-                                     : ((one_point && many) || (grad && reaching >= (double)(1u << 22))) &&
-                                           n_tri >= 4096 && n_tri <= 24576;
+        const bool fans = b->grid_crowd >= 10.0f;
+        const bool walks = (!fans || reaching >= (double)(1u << 23)) &&
+                           (electrons ? n_tri >= 2048 && n_tri <= 49152
+                                      : ((one_point && many) || (grad && reaching >= (double)(1u << 22))) &&
+                                            n_tri >= 4096 && n_tri <= 24576);
         p->P.grid = walks ? grid_of(b, p->inst.data(), n_inst, 1) : dev::GridSet{};
         int pencils = 0;                // looked at; a plan of more than eight takes the trees
         for (int i = 0; i < n_inst && p->P.grid.desc; ++i) {

@@ -35,10 +35,10 @@ def revolved(n, profile):
     return np.array(xyz), np.array(tri, np.int32)
 
 
-def solids(parts, active):
+def solids(parts, active, turn=TILT):
     xyz, tri, solid, base = [], [], [], 0
     for s, (x, t) in enumerate(parts):
-        xyz.append(x @ TILT.T)
+        xyz.append(x @ turn.T)
         tri.append(t + base)
         solid.append(np.full(len(t), s, np.int32))
         base += len(x)
@@ -78,3 +78,21 @@ def test_oblique_mesh_on_grids_matches_the_trees():
     assert grids[0] < 1.5 < trees[0]
     assert grids[1] == trees[1] and grids[1][4] == 0
     assert np.array_equal(grids[2], trees[2])
+
+
+@pytest.mark.parametrize("rings,n,e_model,grids", [(True, 6_000_000, 0, True), (False, 6_000_000, 0, False),
+                                                   (False, 60_000_000, 0, True), (True, 2_000_000, 1, True),
+                                                   (False, 2_000_000, 1, False)])
+def test_fans_walk_grids_in_large_runs_only(rings, n, e_model, grids):
+    """A fan's centre is a long list in one cell, which holds up every iteration of a run."""
+    inside = [(r, z) for r in (7.0, 14.0, 22.0) for z in (-60.0,)] if rings else []
+    parts = []
+    for k in range(3):
+        wall = [(30.0 - k, -60.0 + k + (60.0 - 2 * k) * j / 4) for j in range(5)] if rings else [(30.0 - k, -60.0 + k), (30.0 - k, -k)]
+        low, high = [(r - k, -60.0 + k) for r, _ in inside], [(r - k, -k) for r, _ in inside[::-1]]
+        parts.append(revolved(128 if rings else 400, low + wall + high))
+    bvh = api.gadep_bvh_build(solids(parts, [0, 0, 1], np.eye(3)), 0)
+    assert 4096 <= bvh.stats()["n_tri"] <= 24576
+    inst = api.make_instances([(662.0, W.Source(kind=W.SRC_POINT, pos=(1.0, 2.0, 8.0)), n, 0, [])])
+    _, nodes, _, _, tested = api.gadep_count_work(bvh, api.Materials.default(), inst, api.make_opts(variant=2, e_model=e_model))
+    assert (tested < 1.5 * nodes) == grids
