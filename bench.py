@@ -331,10 +331,11 @@ def measure_forms(dev, scale=1.0):
 
 
 def structure_bytes(nodes, boxes, tris):
-    """Algorithmic bytes of the traversal: node and triangle records, or cell words, list
-    entries and triangle records where the run walks grids (each cell counts as one node
-    and one box; a tree's nodes hold two boxes and more)."""
-    if boxes == nodes:
+    """Algorithmic bytes of one run's traversal: node and triangle records, or cell words,
+    list entries and triangle records where the run walks grids (each cell counts as one
+    node and one box, a tree's node as two boxes and more; the few queries that a run on
+    grids leaves to the tree are billed as cells)."""
+    if boxes < 1.5 * nodes:
         return CELL_BYTES * nodes + CELL_TRI_BYTES * tris
     return NODE_BYTES * nodes + TRI_BYTES * tris
 
@@ -603,13 +604,14 @@ def main():
     qlog = [p.queue_sizes() for p in plans]
     queued = sum(sum(q) for q in qlog)      # photons the trace launches of one step served
     # algorithmic work of one step (instrumented copy of the kernel, untimed)
-    nodes = tris = relocated = boxes = 0
+    nodes = tris = relocated = boxes = walked = 0
     for i, E in enumerate(cfg["energies"]):
         _, nv, nt, nr, nb = api.gadep_count_work(bvh, mats, api.make_instances([(E, cfg["src"], n, i, [])]), opts)
         nodes += nv
         tris += nt
         relocated += nr
         boxes += nb
+        walked += structure_bytes(nv, nb, nt)       # each energy is a run of its own form
     flops_per_step = FLOP_PER_BOX * boxes + FLOP_PER_TRI * tris
     # launches and device time per kernel kind over the timed steps
     kstats = {}
@@ -634,9 +636,9 @@ def main():
     # nearest-hit queries: every segment but the one of a history that ends at birth
     # (born in the world aimed away from the scene box), which is counted without a query
     queries = segs - sum(f["culled"] for f in fepe)
-    # algorithmic node and triangle bytes of the traversal (64 B per node visit, 48 B per
-    # triangle test), served by L1 and L2, per second of the dominant kernel
-    l1l2_gbs = structure_bytes(nodes, boxes, tris) * args.steps / (dom_ms / 1e3) / 1e9
+    # algorithmic node and triangle bytes of the traversal, served by L1 and L2, per second
+    # of the dominant kernel
+    l1l2_gbs = walked * args.steps / (dom_ms / 1e3) / 1e9
     # the timed plans hold the mesh's cached wavefront buffers; release them so the
     # public-API calls below find the cache free, as a caller's successive runs do
     n_plans, shape = len(plans), plans[0].shape()
