@@ -218,6 +218,15 @@ gadep_status gadep_bvh_build(const detmesh_mesh *m, int32_t device, gadep_bvh **
 gadep_status gadep_bvh_build_opts(const detmesh_mesh *m, const gadep_bvh_opts *opts, int32_t device,
                                   gadep_bvh **out);
 gadep_status gadep_bvh_get_stats(const gadep_bvh *b, gadep_bvh_stats *out);
+
+/* Device memory of the uniform grids that the segment queries of middling meshes walk beside
+ * the trees (no counterpart in the paper), in bytes; 0 where the mesh has none.  Meshes of
+ * 2,048 to 81,920 triangles get them with the device copy, about 3 KB per triangle (20,088
+ * triangles: 63 MB, their trees 4), and building them takes 14 B more per cell for the moment
+ * (146 MB there).  Meshes that they do not suit (triangles mostly as large as the mesh, details
+ * of 10^-5 of its distance from the origin) have none, and none are built where the device has
+ * no room: every run then takes the trees, with the same results. */
+gadep_status gadep_bvh_grid_bytes(const gadep_bvh *b, int64_t *bytes);
 /* Host-side invariant check of every tree, on the decoded (quantised) boxes:
  * each of its triangles held by at least one leaf and never twice by one leaf,
  * every child box non-empty and meeting its parent's, empty slots empty, every
@@ -315,7 +324,8 @@ typedef struct {
     float    group_scale[GADEP_MAX_GROUPS];  /* density scale per group (default 1) */
     int32_t  wf_slots;        /* wavefront variant: photon slots in device memory, 1024..2^26 (0 = from
                                  the run: the smallest power of two >= the histories expected to
-                                 reach the scene, within [2^20, 2^25]; ~220 B each) */
+                                 reach the scene, within [2^20, 2^25]; 224 B each, 272 B with
+                                 e_model 1) */
     int32_t  e_model;         /* charged particles set in motion by photon interactions:
                                  0 (default) deposit their kinetic energy at the interaction point;
                                  1 run straight ahead in the continuous-slowing-down

@@ -181,6 +181,12 @@ class Bvh(_Handle):
         d["opts"] = {k: getattr(s.opts, k) for k, _ in capi.gadep_bvh_opts._fields_}
         return d
 
+    def grid_bytes(self):
+        """Device memory of the mesh's uniform grids (0: none)."""
+        n = C.c_int64()
+        check(capi.load().gadep_bvh_grid_bytes(self._h, C.byref(n)))
+        return n.value
+
     def validate(self):
         check(capi.load().gadep_bvh_validate(self._h))
 

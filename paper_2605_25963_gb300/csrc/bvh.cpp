@@ -787,6 +787,14 @@ extern "C" gadep_status gadep_bvh_get_stats(const gadep_bvh *b, gadep_bvh_stats 
     return GADEP_OK;
 }
 
+extern "C" gadep_status gadep_bvh_grid_bytes(const gadep_bvh *b, int64_t *bytes)
+{
+    gadep::clear_error();
+    if (!b || !bytes) return gadep::fail(GADEP_E_INVAL, "gadep_bvh_grid_bytes: NULL argument");
+    *bytes = (int64_t)b->grid_bytes;
+    return GADEP_OK;
+}
+
 namespace {
 
 struct LeafBox { int32_t id, rec; float lo[3], hi[3]; };   // mesh triangle, its record

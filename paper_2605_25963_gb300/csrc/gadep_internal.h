@@ -114,6 +114,7 @@ struct gadep_bvh {
     // and triangle records, and the cells' lists; null when none were built
     void *d_grid = nullptr, *d_grid_list = nullptr;
     size_t grid_cells = 0, grid_tris = 0;   // byte offsets within d_grid
+    size_t grid_bytes = 0;                  // of both blocks
     float grid_safe = 0.0f;                 // origins the grids serve: components within this
     float grid_crowd = 0.0f;                // length of the list that an entry is in, on average, in the worst grid
 };

@@ -259,6 +259,7 @@ void grid_free(gadep_bvh *b)
     cudaFree(b->d_grid);
     cudaFree(b->d_grid_list);
     b->d_grid = b->d_grid_list = nullptr;
+    b->grid_bytes = 0;
     b->grid_safe = b->grid_crowd = 0.0f;
 }
 
@@ -444,6 +445,7 @@ gadep_status grid_build(gadep_bvh *b)
     b->d_grid_list = list;
     b->grid_cells = o_cells;
     b->grid_tris = o_tris;
+    b->grid_bytes = o_tris + (size_t)nt * 9 * sizeof(float4) + (size_t)entries * sizeof(uint32_t);
     b->grid_safe = (float)safe;
     b->grid_crowd = 0.0f;
     for (size_t r = 0; r + 1 < ng; ++r)             // the grid of every triangle serves few queries

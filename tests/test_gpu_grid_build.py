@@ -96,3 +96,19 @@ def test_fans_walk_grids_in_large_runs_only(rings, n, e_model, grids):
     inst = api.make_instances([(662.0, W.Source(kind=W.SRC_POINT, pos=(1.0, 2.0, 8.0)), n, 0, [])])
     _, nodes, _, _, tested = api.gadep_count_work(bvh, api.Materials.default(), inst, api.make_opts(variant=2, e_model=e_model))
     assert (tested < 1.5 * nodes) == grids
+
+
+def test_grids_report_their_memory():
+    """Cells, lists and three permuted copies of the triangles: the copies are 144 B a triangle,
+    and every region's grid has at least 4 B for each of 2^17 cells but for rounding up."""
+    with_grids = api.gadep_bvh_build(api.detmesh_build(W.COAX_P), 0)
+    n_tri, n_region = with_grids.stats()["n_tri"], with_grids.stats()["n_region"]
+    free = torch.cuda.mem_get_info()[0]
+    other = api.gadep_bvh_build(api.detmesh_build(W.COAX_P), 0)
+    taken = free - torch.cuda.mem_get_info()[0]
+    assert other.grid_bytes() == with_grids.grid_bytes() > 144 * n_tri + 2 * 131072 * n_region
+    st = other.stats()
+    # the mesh's blocks, each rounded up to 2 MB by the allocator
+    assert other.grid_bytes() <= taken <= other.grid_bytes() + st["node_bytes"] + st["tri_bytes"] + 64 * n_tri + (20 << 20)
+    assert api.gadep_bvh_build(api.detmesh_build(W.COAX_P), -1).grid_bytes() == 0
+    assert api.gadep_bvh_build(api.detmesh_build(W.BARE_CYLINDER), 0).grid_bytes() == 0
