@@ -465,7 +465,6 @@ dev::GridSet grid_set(const gadep_bvh *b)
     g.list = (const uint32_t *)b->d_grid_list;
     g.n_tri = b->geo.n_tri();
     g.all = (int)(b->regions.size() / 4);
-    g.safe = b->grid_safe;
     return g;
 }
 

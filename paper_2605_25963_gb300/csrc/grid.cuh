@@ -18,7 +18,7 @@
 //
 // Robustness: a triangle is listed in every cell that it meets when the cell is grown
 // by kGridPad of its size on all sides, which exceeds the rounding of the positions
-// computed here for origins within GridSet::safe of the coordinate origin (callers
+// computed here for origins within gadep_bvh::grid_safe of the coordinate origin (callers
 // use the tree beyond that).  The cell indices are carried as exact small floats and
 // only ever move forward, by at least one cell per step, and no step passes the
 // border layer, so a walk ends after at most nx + ny + nz steps.
@@ -43,7 +43,6 @@ struct GridSet {
     const float4 *tris;       // [3][n_tri][3]
     int n_tri;
     int all;                  // grid of every triangle
-    float safe;               // origins within this of the coordinate origin, per component
 };
 
 // One walk: per axis mirrored so that the ray moves towards larger cells.

@@ -48,9 +48,6 @@ namespace gadep {
 gadep_status build_bvh_host(const detmesh_mesh *m, const gadep_bvh_opts &o, gadep_bvh *out);
 
 namespace dev {
-// EM: charged-particle tracks (e_model 1), a separate instantiation so that the
-// photon-only kernels keep their registers.  GRID: the queries walk the regions'
-// grids (grid.cuh) instead of their trees.
 // Source point and direction of a history (the first words of its stream).
 __device__ __forceinline__ void birth(const InstDev &I, Stream &rng, uint32_t k0, uint32_t k1, float &ox, float &oy,
                                       float &oz, float &dx, float &dy, float &dz)
@@ -92,6 +89,11 @@ static __device__ __noinline__ bool birth_reaches(const InstDev *I, unsigned lon
 }
 
 constexpr int kMaxChunk = 256;
+// GRAD: scores of the density groups.  COUNT: the traversal's work.  EM: charged-particle
+// tracks (e_model 1), a separate instantiation so that the photon-only kernels keep their
+// registers.  GRID: the queries walk the regions' grids (grid.cuh) instead of their trees.
+// SCAN: a warp's lanes look together for histories that reach the scene (scans(); not with
+// GRAD or COUNT, and every source lies outside the solids).
 template <bool GRAD, bool COUNT, bool EM, bool GRID, bool SCAN>
 // 4 blocks of 256 threads per SM (64 registers): measured faster than 2 or 3
 // blocks despite the register spills, as the traversal is latency bound.
@@ -177,9 +179,9 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                 const uint32_t take = (uint32_t)min(min(pool_end, s_end[pool_inst]) - pool_next, 32ull);
                 const unsigned long long g = pool_next + lane;
                 bool reaches = lane < take;
-                if (reaches && I->birth_region == 0) {
-                    // Born in the world and aimed away from every solid: the one segment
-                    // of this history escapes with nothing deposited.
+                if (reaches) {
+                    // Aimed away from every solid: the one segment of this history
+                    // escapes with nothing deposited.
                     reaches = birth_reaches(I, g - (pool_inst ? s_end[pool_inst - 1] : 0ull), k0, k1,
                                             make_float3(P.root_lo[0], P.root_lo[1], P.root_lo[2]),
                                             make_float3(P.root_hi[0], P.root_hi[1], P.root_hi[2]));
@@ -208,8 +210,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P, unsig
                 has_sec = false;
                 edep = dep_all = esc = 0.0f;
                 herr = 0u;
-#pragma unroll
-                for (int g = 0; g < (GRAD ? 4 : 1); ++g) score[g] = 0.0f;
+                score[0] = 0.0f;
                 lam = -logf(rng.u01(k0, k1));
                 busy = true;
             }
@@ -1178,13 +1179,12 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
     const bool wf_ok = n_inst <= kWavefrontMaxInstances &&
                        wavefront_supports((int)(regions.size() / 4), (long long)b->geo.n_tri());
     // The wavefront form has a fixed cost per run (~2.5 ms: slot set, iterations of
-    // small queues) and ~1.5 ns per history that reaches the scene; the megakernel
-    // ~1 ms and ~6.7 ns (coax and Table 4 detector at 2e6 .. 1e7 histories per run):
-    // break-even near 2.9e5 reaching histories.  Histories that miss the scene cost
-    // little in either form.
-    // (With grids and chunks by what is left the megakernel is the faster one up to about
-    // 1e6: 2e6 coax histories, 5e5 reaching, 2.3 / 3.7 ms.  The line stays, since the two
-    // forms differ in about one history in a million, and so would a call's results.)
+    // small queues) and ~1.5 ns per history that reaches the scene; histories that miss
+    // it cost little in either form.  The line, 2^18 reaching histories, was drawn where the
+    // megakernel on trees broke even (~1 ms and ~6.7 ns).  On grids and with chunks by what is
+    // left it is the faster form up to about 1e6: 2e6 coax histories, 5e5 reaching, 2.3 / 3.7
+    // ms, 5e5 of a volume source 1.3 / 3.7.  The line stays all the same, since the two forms
+    // differ in about one history in a million, and so would a call's results.
     if (variant == GADEP_VARIANT_AUTO)
         variant = wf_ok && reaching >= (double)(1u << 18) ? GADEP_VARIANT_WAVEFRONT : GADEP_VARIANT_MEGA;
     if (variant == GADEP_VARIANT_WAVEFRONT && !wf_ok) {
@@ -1209,8 +1209,11 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
         // 2.4e6 5.59 / 5.67; with charged-particle tracks, 1.25e6 reaching 8.3 / 5.8, 3e5
         // reaching 5.9 / 4.2 (3,456 triangles 7.0 / 5.0).  On the smallest meshes
         // the tree is a few nodes (192 triangles 2.80 / 3.37), on large ones the cells miss
-        // the caches (25,112 triangles, 1.5e6 reaching 5.38 / 5.52; 76,280 triangles, 7.5e6
-        // reaching 14.5 / 15.8); a plain volume source gains 2 % at best.
+        // the caches (76,280 triangles, 7.5e6 reaching 14.5 / 15.8); a plain volume source
+        // gains 2 % at best.  The end at 24,576 is a compromise, for the size at which the
+        // cells miss depends on the run too: 26,520 triangles at 1332 keV, 1.1e6 reaching 4.96 /
+        // 5.43, 5e6 10.3 / 10.0, 2.5e7 36.3 / 33.9; 55,800 triangles 5.41 / 6.33, 11.2 / 11.8,
+        // 39.0 / 38.5.
         // Where triangles crowd in a few cells (end faces that are fans: 10 and more to a
         // list that an entry is in, on average; rings have 3 to 9) one lane's long list
         // holds up each iteration.  Such meshes need 2^23 that reach: nested cans with fans of
