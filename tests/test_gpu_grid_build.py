@@ -112,3 +112,16 @@ def test_grids_report_their_memory():
     assert other.grid_bytes() <= taken <= other.grid_bytes() + st["node_bytes"] + st["tri_bytes"] + 64 * n_tri + (20 << 20)
     assert api.gadep_bvh_build(api.detmesh_build(W.COAX_P), -1).grid_bytes() == 0
     assert api.gadep_bvh_build(api.detmesh_build(W.BARE_CYLINDER), 0).grid_bytes() == 0
+
+
+def test_many_small_solids_share_the_smallest_grids():
+    """2^22 cells for the smallest grids together, twice that with borders and rounding up, and
+    160 cells a triangle for those of the world and of every triangle."""
+    parts = []
+    for k in range(150):
+        xyz, tri = revolved(8, [(3.0, 0.0), (3.0, 6.0)])
+        parts.append((xyz + 8.0 * np.array([k % 5, k // 5 % 5, k // 25]), tri))
+    bvh = api.gadep_bvh_build(solids(parts, [1] * 150), 0)
+    n_tri = bvh.stats()["n_tri"]
+    assert n_tri >= 2048
+    assert 0 < bvh.grid_bytes() <= 4 * (2 * (1 << 22) + 2 * 2 * 160 * n_tri) + 4 * 3 * 1000 * n_tri
