@@ -125,3 +125,16 @@ def test_many_small_solids_share_the_smallest_grids():
     n_tri = bvh.stats()["n_tri"]
     assert n_tri >= 2048
     assert 0 < bvh.grid_bytes() <= 4 * (2 * (1 << 22) + 2 * 2 * 160 * n_tri) + 4 * 3 * 1000 * n_tri
+
+
+@pytest.mark.parametrize("shape", ["boxes", "tilted boxes"])
+def test_flat_meshes_have_no_grids(shape):
+    """Boxes along the axes are the trees' best case."""
+    parts = []
+    for k in range(8):
+        xyz, tri = box((0.0, 0.0, 0.0), (8.0, 8.0, 8.0), 6)
+        xyz = np.round(xyz / (8.0 / 6)) * (8.0 / 6)             # without the dents
+        parts.append((xyz + 10.0 * np.array([k & 1, k >> 1 & 1, k >> 2]), tri))
+    bvh = api.gadep_bvh_build(solids(parts, [1] * 8, np.eye(3) if shape == "boxes" else TILT), 0)
+    assert bvh.stats()["n_tri"] == 8 * 432
+    assert (bvh.grid_bytes() > 0) == (shape == "tilted boxes")

@@ -19,13 +19,18 @@ NEAR, FAR = (W.Source(kind=W.SRC_POINT, pos=(0.0, 0.0, z)) for z in (60.0, 3e6))
 
 
 def box(lo, hi, n):
-    """A closed box of n x n squares a face: (xyz, tri)."""
+    """A closed box of n x n squares a face: (xyz, tri).  The vertices within the faces at both
+    ends of y and the lower end of z lie 0.02 inside by turns, for flat meshes have no grids."""
     at, xyz, tri = {}, [], []
 
     def vertex(p):
         if p not in at:
             at[p] = len(xyz)
-            xyz.append([lo[a] + (hi[a] - lo[a]) * p[a] / n for a in range(3)])
+            q = [lo[a] + (hi[a] - lo[a]) * p[a] / n for a in range(3)]
+            for a, side, move in ((1, 0, 0.02), (1, n, -0.02), (2, 0, 0.02)):
+                if p[a] == side and sum(p) % 2 and all(0 < p[b] < n for b in range(3) if b != a):
+                    q[a] += move
+            xyz.append(q)
         return at[p]
 
     for a in range(3):
