@@ -970,6 +970,18 @@ dev::GridSet grid_of(const gadep_bvh *b, const dev::InstDev *inst, int n_inst, i
     return g;
 }
 
+// Solids within one another, at most: the shells that a photon crosses one after another.
+int nest_depth(const MeshData &m)
+{
+    int deepest = 0;
+    for (int32_t s = 0; s < m.n_solid(); ++s) {
+        int depth = 0;
+        for (int32_t p = s; p >= 0; p = m.solids[p].parent) ++depth;
+        deepest = std::max(deepest, depth);
+    }
+    return deepest;
+}
+
 // Whether a pencil's ray passes through an edge or a vertex of the mesh, within the rounding
 // of the FP32 edge functions (or lies in the plane of a triangle).  Its photons then meet two
 // surfaces at one distance again and again, and a walk of the grids only precedes the tree's
@@ -1219,11 +1231,18 @@ gadep_status plan_create(const gadep_bvh *b, const gadep_materials *mat, int32_t
         // holds up each iteration.  Such meshes need 2^23 that reach: nested cans with fans of
         // 256, 1.1e6 reaching 6.19 / 7.50, 3e6 10.0 / 10.8, 1e7 23.9 / 18.2; one can with fans
         // of 1,200, 1.8e6 reaching 9.4 / 14.4, 6e6 21.1 / 20.3; with tracks 1.8e5 6.7 / 9.5.
-        const int n_tri = b->geo.n_tri();
+        // A walk gains where hops are short, in solids nested in one another: a hop on the
+        // tree is a descent from its root whatever its length.  Trees / grids by the depth
+        // (cylinders of 4,352 to 17,408 triangles; 1.5e6 reaching at 1332 keV, 2e7 reaching,
+        // with tracks 5e6 histories): one 0.79, 0.99, 0.85; two 0.77 - 0.81, 1.05 - 1.10, 0.89 -
+        // 0.97; four 0.90 - 0.91, 1.05 - 1.21, 1.23; six (coaxes) 1.01 - 1.05, 1.07 - 1.13, 1.31 -
+        // 1.48; eight 1.25, 1.41, 1.99.
+        const int n_tri = b->geo.n_tri(), nest = nest_depth(b->geo);
         const bool fans = b->grid_crowd >= 10.0f;
-        const bool walks = (!fans || reaching >= (double)(1u << 23)) &&
+        const bool walks = nest >= 4 && (!fans || reaching >= (double)(1u << 23)) &&
                            (electrons ? n_tri >= 2048 && n_tri <= 49152
-                                      : ((one_point && many) || (grad && reaching >= (double)(1u << 22))) &&
+                                      : ((one_point && reaching >= (double)(nest >= 5 ? 1u << 20 : 1u << 22)) ||
+                                         (grad && reaching >= (double)(1u << 22))) &&
                                             n_tri >= 4096 && n_tri <= 24576);
         p->P.grid = walks ? grid_of(b, p->inst.data(), n_inst, 1) : dev::GridSet{};
         int pencils = 0;                // looked at; a plan of more than eight takes the trees

@@ -87,11 +87,11 @@ def test_fans_walk_grids_in_large_runs_only(rings, n, e_model, grids):
     """A fan's centre is a long list in one cell, which holds up every iteration of a run."""
     inside = [(r, z) for r in (7.0, 14.0, 22.0) for z in (-60.0,)] if rings else []
     parts = []
-    for k in range(3):
+    for k in range(5):
         wall = [(30.0 - k, -60.0 + k + (60.0 - 2 * k) * j / 4) for j in range(5)] if rings else [(30.0 - k, -60.0 + k), (30.0 - k, -k)]
         low, high = [(r - k, -60.0 + k) for r, _ in inside], [(r - k, -k) for r, _ in inside[::-1]]
-        parts.append(revolved(128 if rings else 400, low + wall + high))
-    bvh = api.gadep_bvh_build(solids(parts, [0, 0, 1], np.eye(3)), 0)
+        parts.append(revolved(100 if rings else 400, low + wall + high))
+    bvh = api.gadep_bvh_build(solids(parts, [0, 0, 0, 0, 1], np.eye(3)), 0)
     assert 4096 <= bvh.stats()["n_tri"] <= 24576
     inst = api.make_instances([(662.0, W.Source(kind=W.SRC_POINT, pos=(1.0, 2.0, 8.0)), n, 0, [])])
     _, nodes, _, _, tested = api.gadep_count_work(bvh, api.Materials.default(), inst, api.make_opts(variant=2, e_model=e_model))
@@ -138,3 +138,20 @@ def test_flat_meshes_have_no_grids(shape):
     bvh = api.gadep_bvh_build(solids(parts, [1] * 8, np.eye(3) if shape == "boxes" else TILT), 0)
     assert bvh.stats()["n_tri"] == 8 * 432
     assert (bvh.grid_bytes() > 0) == (shape == "tilted boxes")
+
+
+@pytest.mark.parametrize("depth,n,e_model,grids", [(1, 6_000_000, 0, False), (3, 2_000_000, 1, False), (4, 2_000_000, 1, True),
+                                                   (4, 6_000_000, 0, False), (4, 12_000_000, 0, True), (5, 6_000_000, 0, True)])
+def test_wavefront_runs_walk_grids_in_deep_nests(depth, n, e_model, grids):
+    """Half of the histories reach the can below the source."""
+    parts = []
+    for k in range(depth):
+        r, top, low = 30.0 - k, -float(k), -60.0 + k
+        rings = [0.25 * r, 0.5 * r, 0.75 * r]
+        parts.append(revolved(300 if depth == 1 else 100, [(x, low) for x in rings] +
+                              [(r, low + (top - low) * j / 4) for j in range(5)] + [(x, top) for x in rings[::-1]]))
+    bvh = api.gadep_bvh_build(solids(parts, [0] * (depth - 1) + [1], np.eye(3)), 0)
+    assert 4096 <= bvh.stats()["n_tri"] <= 24576 and bvh.grid_bytes() > 0
+    inst = api.make_instances([(662.0, W.Source(kind=W.SRC_POINT, pos=(1.0, 2.0, 3.0)), n, 0, [])])
+    _, nodes, _, _, tested = api.gadep_count_work(bvh, api.Materials.default(), inst, api.make_opts(variant=2, e_model=e_model))
+    assert (tested < 1.5 * nodes) == grids

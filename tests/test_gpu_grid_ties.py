@@ -67,9 +67,11 @@ def nested(parts, active):
 
 
 def box_in_a_box(swap):
-    """A dead Ge box and an active one within it that shares the middle of its top face."""
+    """A dead Ge box and an active one within it that shares the middle of its top face, within
+    two shells."""
     outer, inner = box((-8.0, -8.0, -16.0), (8.0, 8.0, 0.0), 16), box((-4.0, -4.0, -8.0), (4.0, 4.0, 0.0), 8)
-    return nested([inner, outer], [1, 0]) if swap else nested([outer, inner], [0, 1])
+    shells = [box((-8.0 - d, -8.0 - d, -16.0 - d), (8.0 + d, 8.0 + d, d), 4) for d in (2.0, 1.0)]
+    return nested(shells + [inner, outer], [0, 0, 1, 0]) if swap else nested(shells + [outer, inner], [0, 0, 0, 1])
 
 
 def boxes_on_an_edge(n, swap):
