@@ -194,8 +194,9 @@ struct STally {
 // histories' deposits, coax, rms of 12 runs, trace on trees with FP32 / on grids with FP32 /
 // on grids with FP64: 1e8 histories at 1332 keV 1.2e-9 / 2.2e-9 / 1.0e-10, 1e7 at 662 keV
 // 0.7e-9 / 1.5e-9 / 1.6e-10, with charged-particle tracks 1.1e-9 / 1.4e-9 / 0.4e-9 (physics of
-// 1e8 histories on grids 2.94 -> 3.10 ms).  Gradients, 6e6 histories: 1.7e-9 / 4.8e-9 / 2.1e-9
-// (physics 2.08 -> 1.99 ms; every lane adding in FP64 3.62).
+// 1e8 histories on grids 2.94 -> 3.10 ms).  Gradients of 3e6 histories at 1332 keV, FP32 a
+// history at a time on trees / FP64 2.2e-9 / 2.8e-10 (physics of 1.2e7 2.08 -> 1.99 ms; every
+// lane adding in FP64 3.62).
 template <bool GRAD, bool WIDE>
 struct BlockTally {
     using Tally = STally<WIDE>;
