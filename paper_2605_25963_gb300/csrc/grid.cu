@@ -67,10 +67,10 @@ __host__ __device__ inline uint32_t padded(uint32_t c) { return (c + (c >= kLong
 // list null: counts[cell] += 1 per triangle that meets it; otherwise the ids go to
 // list[start[cell] + counts[cell]++] (behind the length where the cell has kLong or more).
 // One kernel for both, so that both find the same cells to the last bit.
-// In FP32 and cells, with the triangle's lowest cell as the origin: coordinates of at most 160
-// are then good to 2e-5 of a cell, and kSlack more than covers the tests' rounding (the
-// normal's, which a sliver's cancels, is added by itself): 0.2 % more cells than in FP64, none
-// fewer.  Bound by issue, 2.5e11 cells of boxes a second.  FP64 throughout, a triangle to a
+// In FP32 and cells, with the triangle's lowest cell as the origin: coordinates of 160 are then
+// good to 1e-5 of a cell, of 16,000 (the longest a thin region can be) to 1e-3, and kSlack and
+// kGridPad cover that and the tests' rounding (the normal's, which a sliver's cancels, is added
+// by itself): 0.2 % more cells than in FP64, none fewer.  Bound by issue, 2.5e11 cells of boxes a second.  FP64 throughout, a triangle to a
 // warp, took 2.8 ms a pass on 3,456 triangles, most of it one warp with the largest box, and
 // 3.1 on 20,088: now 0.14 and 0.29 (counting), 0.22 and 0.36 (lists).
 constexpr float kSlack = 1e-3f;
@@ -274,7 +274,8 @@ void grid_free(gadep_bvh *b)
 
 // Builds the grids of b (device current).  Where they do not suit the mesh (coordinates
 // too coarse for the cells' margin, lists too long for the cell words, too few or too many
-// triangles, mostly flat or as large as the grids) or leave no memory, the tree serves alone; b->d_grid stays null.
+// triangles, mostly flat or as large as the grids) or leave no memory, the tree serves
+// alone; b->d_grid stays null.
 gadep_status grid_build(gadep_bvh *b)
 {
     const MeshData &m = b->geo;

@@ -49,6 +49,18 @@ def test_long_lists(e_model):
     assert np.array_equal(grids[2], trees[2])
 
 
+def test_a_long_thin_rod():
+    """Thousands of cells along one axis, two dozen across."""
+    rod = revolved(64, [(0.25, -70.0)] + [(0.5, -70.0 + 120.0 * k / 70) for k in range(71)] + [(0.25, 50.0)])
+    bvh = api.gadep_bvh_build(solids([rod], [1], np.eye(3)), 0)
+    assert bvh.stats()["n_tri"] >= 8192
+    src = W.Source(kind=W.SRC_DISK, pos=(0.1, 0.2, 51.0), radius=0.6)
+    grids, trees = on_grids_and_on_trees(bvh, src, 122.0, 500_000, variant=MEGA)
+    assert grids[0] < 1.5 < trees[0]
+    assert grids[1] == trees[1] and grids[1][4] == 0
+    assert np.array_equal(grids[2], trees[2])
+
+
 def test_megakernel_gradients_on_grids_match_the_trees():
     bvh = api.gadep_bvh_build(api.detmesh_build(W.GRAD_DET), 0)
     mats, out = api.Materials.default(), []
